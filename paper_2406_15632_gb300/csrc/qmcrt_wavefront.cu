@@ -5,12 +5,12 @@
 // but from the second order on each lane scatters into its own direction and the warp
 // waits for its longest walk.  Here every order is a launch over the packets still
 // alive, and between orders the live packets are regrouped by a key built from their
-// position (one of 16^3 cells of the box) and their new direction (32 bins in cos theta
+// position (up to 16^3 cells of the box) and their new direction (up to 32 bins in cos theta
 // x 64 in phi), so a warp again traces 32 similar rays:
 //
 //   order 1:   emission, forced step, peel-off, roulette, scattering for order 2 ->
 //              queue (with each packet's key, counted in the bucket histogram)
-//   order k:   bucket offsets (a tiled scan) -> record indices into
+//   order k:   bucket cursors -> record indices into
 //              buckets -> forced step (or march), peel-off, roulette, scattering for
 //              k+1 -> the other queue
 //
@@ -30,19 +30,19 @@ namespace qmcrt {
 
 namespace {
 
-// Key split measured on the clumpy envelope (2^24 packets, 20 orders): 16^3 position
-// cells with 32 x 64 direction bins (2^23 buckets, position-major) take 77 ms, against
-// 89 ms for the octant with the same direction bins (2^14 buckets) and 80 ms for 8^3
-// cells; finer direction bins or position cells gain nothing more (77-79 ms), 2^25 buckets
-// lose it again to the histogram's clearing and scan (83 ms).  Packets that start close
-// together in nearly one direction cross nearly the same cells, so a warp's loads share
-// cache lines.
-constexpr int WV_POS_BITS = 4;  // per axis: 16 position cells
-constexpr int WV_COS_BITS = 5;  // direction bins: 32 in cos theta
-constexpr int WV_PHI_BITS = 6;  //                 x 64 in phi
-constexpr int WV_KEY_BITS = 3 * WV_POS_BITS + WV_COS_BITS + WV_PHI_BITS;
-constexpr int WV_BUCKETS = 1 << WV_KEY_BITS;
-static_assert(WV_KEY_BITS >= 20 && WV_KEY_BITS <= 30, "the scan takes 1024-bucket tiles, their totals in one block");
+// The regrouping key: position cells of the box, 2^pos per axis, then direction bins, 2^cos in
+// cos theta and 2^phi in phi; position-major, so that packets that start close together in
+// nearly one direction, which cross nearly the same cells, are traced by one warp and share
+// cache lines.  The finest split suits the largest queues; the buckets are cleared and
+// scanned once an order whatever the queue holds, so a smaller one takes fewer (wave_bits).
+struct WaveKey {
+    int pos, cos, phi;  // bits
+    int shift;          // low bits of the key dropped (queues too small to hold the cursors)
+};
+constexpr int WV_MAX_BITS = 23, WV_MAX_BUCKETS = 1 << WV_MAX_BITS;
+constexpr int WV_TAIL_BYTES = WV_MAX_BUCKETS / 256;  // counters, behind the histogram
+
+__host__ __device__ constexpr int key_bits(const WaveKey &K) { return 3 * K.pos + K.cos + K.phi - K.shift; }
 
 template <class T>
 struct Packet {
@@ -59,13 +59,20 @@ struct alignas(16) Rec {
 };
 static_assert(sizeof(Rec<float>) == 64 && sizeof(Rec<double>) == 128, "record size");
 
+// Counters of one order: packets appended for it, its chunk counter, its bucket space taken.
+struct WaveCount {
+    uint32_t live, chunk, space, pad;
+};
+static_assert(66 * sizeof(WaveCount) <= WV_TAIL_BYTES, "counters of every order (at most 64) and one more");
+
 template <class T>
 struct WaveWork {
     Rec<T> *q[2];       // [cap] each: order k reads q[(k + 1) & 1] and appends to q[k & 1]
-    uint32_t *count;    // [3] packets of this order, packets appended for the next, chunk counter
+    WaveCount *count;   // [order]
     uint32_t *keys;     // [cap] bucket of each appended record
     uint32_t *perm;     // [cap] record indices of the queue being read, in bucket order
-    uint32_t *hist;     // [WV_BUCKETS] histogram of the appended records, then bucket cursors
+    uint32_t *hist;     // [buckets] histogram of the appended records
+    WaveKey key;
 };
 
 template <class T>
@@ -78,24 +85,25 @@ __device__ __forceinline__ void copy_rec(Rec<T> *dst, const Rec<T> *src)
 }
 
 template <class T>
-__device__ __forceinline__ uint32_t wave_key(const MediumP<T> &G, const T pos[3], const T n[3])
+__device__ __forceinline__ uint32_t wave_key(const MediumP<T> &G, const WaveKey &K, const T pos[3], const T n[3])
 {
-    constexpr int NP = 1 << WV_POS_BITS, NC = 1 << WV_COS_BITS, NF = 1 << WV_PHI_BITS;
+    const int NP = 1 << K.pos, NC = 1 << K.cos, NF = 1 << K.phi;
     uint32_t key = 0;
     for (int c = 0; c < 3; ++c) {
         const T f = (pos[c] - G.lo[c]) / (G.hi[c] - G.lo[c]) * T(NP);
-        key = (key << WV_POS_BITS) | (uint32_t)min(NP - 1, max(0, (int)f));
+        key = (key << K.pos) | (uint32_t)min(NP - 1, max(0, (int)f));
     }
-    const int ct = min(NC - 1, max(0, (int)((n[2] + T(1)) * T(NC / 2.0))));
+    const int ct = min(NC - 1, max(0, (int)((n[2] + T(1)) * T(NC) * T(0.5))));
     const float ph = atan2f((float)n[1], (float)n[0]);  // the key only orders packets
-    const int pb = min(NF - 1, max(0, (int)((ph + 3.14159265f) * (float)(NF / 6.283185307179586))));
-    return (key << (WV_COS_BITS + WV_PHI_BITS)) | (uint32_t)(ct << WV_PHI_BITS) | (uint32_t)pb;
+    const int pb = min(NF - 1, max(0, (int)((ph + 3.14159265f) * ((float)NF * 0.159154943f))));
+    return ((key << (K.cos + K.phi)) | (uint32_t)(ct << K.phi) | (uint32_t)pb) >> K.shift;
 }
 
-// Append the lanes with `keep` to queue dst with their bucket keys and count them in
-// the histogram of the next sort (one queue atomic per warp).  All 32 lanes call.
+// Append the lanes with `keep` to queue dst, the queue of order k + 1, with their bucket keys
+// and count them in the histogram of the next sort (one queue atomic per warp).  All 32 lanes
+// call.
 template <class T>
-__device__ __forceinline__ void append(const TraceP<T> &P, const WaveWork<T> &W, Rec<T> *dst, bool keep,
+__device__ __forceinline__ void append(const TraceP<T> &P, const WaveWork<T> &W, int k, Rec<T> *dst, bool keep,
                                        const Packet<T> &p, uint32_t j)
 {
     const unsigned m = __ballot_sync(FULL_MASK, keep);
@@ -103,9 +111,9 @@ __device__ __forceinline__ void append(const TraceP<T> &P, const WaveWork<T> &W,
     const int lane = threadIdx.x & 31;
     const int first = __ffs(m) - 1;
     uint32_t base = 0;
-    if (lane == first) base = atomicAdd(W.count + 1, (uint32_t)__popc(m));
+    if (lane == first) base = atomicAdd(&W.count[k + 1].live, (uint32_t)__popc(m));
     base = __shfl_sync(FULL_MASK, base, first);
-    const uint32_t key = keep ? wave_key(P.med, p.pos, p.n) : 0xffffffffu;
+    const uint32_t key = keep ? wave_key(P.med, W.key, p.pos, p.n) : 0xffffffffu;
     // lanes with equal keys count into the histogram with one atomic (a warp's
     // packets come from one bucket of the last sort and mostly share their key)
     const unsigned peers = __match_any_sync(FULL_MASK, key);
@@ -114,7 +122,7 @@ __device__ __forceinline__ void append(const TraceP<T> &P, const WaveWork<T> &W,
         Rec<T> r;
         r.p = p;
         r.j = j;
-        for (int k = 0; k < (int)(sizeof(r.pad) / 4); ++k) r.pad[k] = 0u;
+        for (int c = 0; c < (int)(sizeof(r.pad) / 4); ++c) r.pad[c] = 0u;
         copy_rec(dst + q, &r);
         W.keys[q] = key;
         if (lane == __ffs(peers) - 1) atomicAdd(W.hist + key, (uint32_t)__popc(peers));
@@ -219,77 +227,79 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_wave_first(cons
         p.S[0] = wgt;
     }
     const bool on = run_order(P, 1, i, live, wd, p);
-    append(P, W, W.q[1], on, p, (uint32_t)j);
+    append(P, W, 1, W.q[1], on, p, (uint32_t)j);
     if (live && !on && P.train_log) write_log(P, i, j, p);
 }
 
-// Exclusive scan of the bucket histogram into cursors, in three launches: each block scans
-// a tile of 1024 buckets in shared memory and records the tile's total; one block scans
-// the totals; every bucket then adds its tile's offset.
-__global__ void __launch_bounds__(1024) k_wave_scan_tiles(uint32_t *hist, uint32_t *tile_sum)
+// Bucket cursors of the queue for order k: every block scans a tile of buckets in order and
+// takes the tile's space from one counter (tiles may end up in any order: only packets of
+// one tile need to be close), clearing the histogram behind it for the next sort.  The cursors
+// lie in the queue that order k will append to.  Bound by the L2 pass over the buckets, of
+// which it writes only those that hold records.
+constexpr int WV_TILE = 4096, WV_PER = WV_TILE / 256;
+__global__ void __launch_bounds__(256) k_wave_cursors(uint32_t *__restrict__ hist, uint32_t *__restrict__ cursor,
+                                                      int buckets, WaveCount *cnt)
 {
-    __shared__ uint32_t s[1024];
-    const int t = threadIdx.x;
-    const size_t b = (size_t)blockIdx.x * 1024 + t;
-    const uint32_t x = hist[b];
-    s[t] = x;
+    __shared__ uint32_t s_warp[8], s_base;
+    const int t = threadIdx.x, lane = t & 31;
+    const int b0 = blockIdx.x * WV_TILE + t * WV_PER;
+    uint4 v[WV_PER / 4];
+    uint32_t sum = 0;
+#pragma unroll
+    for (int q = 0; q < WV_PER / 4; ++q) {
+        v[q] = b0 + 4 * q < buckets ? *reinterpret_cast<const uint4 *>(hist + b0 + 4 * q) : make_uint4(0, 0, 0, 0);
+        sum += v[q].x + v[q].y + v[q].z + v[q].w;
+    }
+    uint32_t run = sum;  // inclusive over the warp
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(FULL_MASK, run, o);
+        if (lane >= o) run += x;
+    }
+    if (lane == 31) s_warp[t >> 5] = run;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const uint32_t v = t >= off ? s[t - off] : 0u;
-        __syncthreads();
-        s[t] += v;
-        __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        if (w < (t >> 5)) before += s_warp[w];
+        all += s_warp[w];
     }
-    hist[b] = s[t] - x;
-    if (t == 1023) tile_sum[blockIdx.x] = s[1023];
-}
-
-// exclusive scan of the n tile totals (n a multiple of 1024), one block
-__global__ void __launch_bounds__(1024) k_wave_scan_sums(uint32_t *tile_sum, int n)
-{
-    __shared__ uint32_t s[1024];
-    const int t = threadIdx.x, per = n / 1024;
-    uint32_t tot = 0;
-    for (int q = 0; q < per; ++q) tot += tile_sum[t * per + q];
-    s[t] = tot;
+    if (t == 0) s_base = all ? atomicAdd(&cnt->space, all) : 0u;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const uint32_t v = t >= off ? s[t - off] : 0u;
-        __syncthreads();
-        s[t] += v;
-        __syncthreads();
+    if (!sum) return;  // empty buckets have no record to place
+    run += s_base + before - sum;
+#pragma unroll
+    for (int q = 0; q < WV_PER / 4; ++q) {
+        const uint4 x = v[q];
+        if (!(x.x | x.y | x.z | x.w)) continue;
+        uint4 c;
+        c.x = run;
+        c.y = c.x + x.x;
+        c.z = c.y + x.y;
+        c.w = c.z + x.z;
+        run = c.w + x.w;
+        *reinterpret_cast<uint4 *>(cursor + b0 + 4 * q) = c;
+        *reinterpret_cast<uint4 *>(hist + b0 + 4 * q) = make_uint4(0, 0, 0, 0);
     }
-    uint32_t run = s[t] - tot;
-    for (int q = 0; q < per; ++q) {
-        const uint32_t x = tile_sum[t * per + q];
-        tile_sum[t * per + q] = run;
-        run += x;
-    }
-}
-
-__global__ void __launch_bounds__(1024) k_wave_scan_add(uint32_t *hist, const uint32_t *tile_sum)
-{
-    hist[(size_t)blockIdx.x * 1024 + threadIdx.x] += tile_sum[blockIdx.x];
 }
 
 // Bucket order of the appended records: perm[cursor of its key] = record index, one
 // cursor atomic per run of equal keys in a warp.
-template <class T>
-__global__ void __launch_bounds__(256) k_wave_scatter(WaveWork<T> W)
+__global__ void __launch_bounds__(256) k_wave_scatter(const uint32_t *__restrict__ keys, uint32_t *__restrict__ cursor,
+                                                      uint32_t *__restrict__ perm, const WaveCount *__restrict__ cnt)
 {
-    const uint32_t n = W.count[1];
+    const uint32_t n = cnt->live;
     const int lane = threadIdx.x & 31;
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t q0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); q0 < n; q0 += stride) {  // uniform per warp
         const uint32_t q = q0 + lane;
         const bool v = q < n;
-        const uint32_t key = v ? W.keys[q] : 0xffffffffu;
+        const uint32_t key = v ? keys[q] : 0xffffffffu;
         const unsigned peers = __match_any_sync(FULL_MASK, key);
         const int leader = __ffs(peers) - 1;
         uint32_t base = 0;
-        if (v && lane == leader) base = atomicAdd(W.hist + key, (uint32_t)__popc(peers));
+        if (v && lane == leader) base = atomicAdd(cursor + key, (uint32_t)__popc(peers));
         base = __shfl_sync(FULL_MASK, base, leader);
-        if (v) W.perm[base + __popc(peers & ((1u << lane) - 1u))] = q;
+        if (v) perm[base + __popc(peers & ((1u << lane) - 1u))] = q;
     }
 }
 
@@ -299,7 +309,7 @@ __global__ void __launch_bounds__(256) k_wave_scatter(WaveWork<T> W)
 template <class T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_wave_order(const __grid_constant__ TraceP<T> P, int k, WaveWork<T> W)
 {
-    const uint32_t n = W.count[0];
+    const uint32_t n = W.count[k].live;
     const int lane = threadIdx.x & 31;
     Rec<T> *const src = (k & 1) ? W.q[0] : W.q[1];  // selects, not an indexed parameter array
     Rec<T> *const dst = (k & 1) ? W.q[1] : W.q[0];
@@ -308,7 +318,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_wave_order(cons
     // so the counter, which passes n by at most two chunks per warp, cannot wrap)
     auto claim = [&]() {
         uint32_t c = 0;
-        if (lane == 0) c = atomicAdd(W.count + 2, 32u);
+        if (lane == 0) c = atomicAdd(&W.count[k].chunk, 32u);
         return __shfl_sync(FULL_MASK, c, 0);
     };
     uint32_t q0 = claim();
@@ -331,7 +341,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_wave_order(cons
         const uint64_t i = P.first + r.j;
         const T wd = live ? point<T>(P.pts, i, 4 * (k - 1) + 2) : T(0);
         const bool on = run_order(P, k, i, live, wd, r.p);
-        append(P, W, dst, on, r.p, r.j);
+        append(P, W, k, dst, on, r.p, r.j);
         if (live && !on && P.train_log) write_log(P, i, r.j, r.p);
         q0 = q1;
     }
@@ -349,11 +359,25 @@ WaveWork<T> carve(void *ws, uint64_t cap)
     };
     W.q[0] = (Rec<T> *)take(cap * sizeof(Rec<T>));
     W.q[1] = (Rec<T> *)take(cap * sizeof(Rec<T>));
-    W.count = (uint32_t *)take(3 * 4);
+    take(12);
     W.keys = (uint32_t *)take(cap * 4);
     W.perm = (uint32_t *)take(cap * 4);
-    W.hist = (uint32_t *)take(WV_BUCKETS * 4 + WV_BUCKETS / 256);
+    W.hist = (uint32_t *)take(WV_MAX_BUCKETS * 4 + WV_TAIL_BYTES);
+    W.count = (WaveCount *)(W.hist + WV_MAX_BUCKETS);
     return W;
+}
+
+// Bits of the key for n packets.  20-order clumpy envelope, 16^3 position cells x 32 x 64 direction
+// bins against 8^3 cells with the same bins: 20.9 / 21.3 ms at 2^22 packets, 6.51 / 6.40 at
+// 2^20, 2.75 / 2.69 at 2^18, 1.79 / 1.73 at 2^16, and on a 32^3 grid 5.49 / 5.18 at 2^20; fewer
+// direction bins lose at every size but the smallest, where no split matters (2^12: 1.15 ms).
+// With a three-launch scan, clears and copies an order took up to 150 us on the buckets alone,
+// and the same runs 22.3, 8.1, 4.4 and 3.3 ms.
+WaveKey wave_bits(uint64_t n, uint64_t queue_bytes)
+{
+    WaveKey K = {n >= (1ull << 21) ? 4 : 3, 5, 6, 0};
+    while (((uint64_t)4 << key_bits(K)) > queue_bytes) ++K.shift;  // the cursors lie in a queue
+    return K;
 }
 
 template <class T>
@@ -361,8 +385,10 @@ cudaError_t launch_wave(const TraceP<T> &P, void *ws, uint64_t cap, int sms, cud
 {
     if (P.count == 0) return cudaSuccess;
     WaveWork<T> W = carve<T>(ws, cap);
-    cudaError_t e = cudaMemsetAsync(W.count, 0, 3 * sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(W.hist, 0, WV_BUCKETS * sizeof(uint32_t), s);
+    W.key = wave_bits(P.count, cap * sizeof(Rec<T>));
+    const int buckets = 1 << key_bits(W.key);
+    cudaError_t e = cudaMemsetAsync(W.count, 0, WV_TAIL_BYTES, s);
+    if (e == cudaSuccess && P.max_orders > 1) e = cudaMemsetAsync(W.hist, 0, (size_t)buckets * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
     const uint64_t threads = (P.ord.threads + 31) & ~31ull;
     k_wave_first<T><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(P, W);
@@ -371,14 +397,9 @@ cudaError_t launch_wave(const TraceP<T> &P, void *ws, uint64_t cap, int sms, cud
     for (int k = 2; k <= P.max_orders; ++k) {
         // the queue appended by order k - 1 holds order k's packets with their keys and
         // histogram: their indices in bucket order into perm
-        k_wave_scan_tiles<<<WV_BUCKETS / 1024, 1024, 0, s>>>(W.hist, W.hist + WV_BUCKETS);
-        k_wave_scan_sums<<<1, 1024, 0, s>>>(W.hist + WV_BUCKETS, WV_BUCKETS / 1024);
-        k_wave_scan_add<<<WV_BUCKETS / 1024, 1024, 0, s>>>(W.hist, W.hist + WV_BUCKETS);
-        k_wave_scatter<T><<<grid, 256, 0, s>>>(W);
-        if ((e = cudaMemcpyAsync(W.count, W.count + 1, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-            return e;
-        if ((e = cudaMemsetAsync(W.count + 1, 0, 2 * sizeof(uint32_t), s)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(W.hist, 0, WV_BUCKETS * sizeof(uint32_t), s)) != cudaSuccess) return e;
+        uint32_t *cursor = (uint32_t *)W.q[k & 1];
+        k_wave_cursors<<<(buckets + WV_TILE - 1) / WV_TILE, 256, 0, s>>>(W.hist, cursor, buckets, W.count + k);
+        k_wave_scatter<<<grid, 256, 0, s>>>(W.keys, cursor, W.perm, W.count + k);
         k_wave_order<T><<<grid, 256, 0, s>>>(P, k, W);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -391,7 +412,7 @@ uint64_t wavefront_workspace_bytes(uint64_t cap, int precision)
 {
     const uint64_t rec = precision == QMCRT_PREC_F64 ? sizeof(Rec<double>) : sizeof(Rec<float>);
     auto pad = [](uint64_t b) { return (b + 255) & ~255ull; };
-    return 2 * pad(cap * rec) + pad(12) + 2 * pad(cap * 4) + pad(WV_BUCKETS * 4 + WV_BUCKETS / 256);
+    return 2 * pad(cap * rec) + pad(12) + 2 * pad(cap * 4) + pad(WV_MAX_BUCKETS * 4 + WV_TAIL_BYTES);
 }
 
 cudaError_t launch_trace_wavefront_f32(const TraceP<float> &p, void *ws, uint64_t cap, int sms, cudaStream_t s)
