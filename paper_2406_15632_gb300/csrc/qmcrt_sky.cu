@@ -28,11 +28,54 @@ namespace qmcrt {
 
 namespace {
 
-// One pass of the separable maximum filter: out = max over the 2D + 1 values of `in`
-// along axis `ax` around each cell of the grown grid [nz + 2D][ny + 2D][nx + 2D].  In the
-// first pass `in` is the grid itself (read at the offset -D, zero outside it); only values
-// kappa rho > 0 raise the maximum (zero, negative and NaN cells count as empty, as in the
-// padded grid the walk reads).
+// The maximum over 3^3 neighbourhoods (D = 1, every point source) in one pass: a warp takes
+// 32 cells of a row (30 outputs), a thread MAX3_ROWS rows, marching along z with the 3 x 3 maxima
+// of the last two planes: its own rows by loads, the neighbours' columns by shuffles.  Only
+// values kappa rho > 0 raise the maximum (zero, negative and NaN cells count as empty, as in
+// the padded grid the walk reads).  One read of the grid and one write of the grown grid; issue
+// and HBM are close (256^3: 345 us for three separable passes, 67 with one row a thread,
+// 31 now; 20 at the copy rate).
+constexpr int MAX3_ROWS = 4, MAX3_WARPS = 4, MAX3_PLANES = 16;
+__global__ void __launch_bounds__(32 * MAX3_WARPS) k_max_filter3(const float *__restrict__ in, float *__restrict__ out,
+                                                                 int nx, int ny, int nz)
+{
+    const int gx = nx + 2, gy = ny + 2, gz = nz + 2;
+    const int x = (int)blockIdx.x * 30 + (int)threadIdx.x - 1;  // in the grown grid; its cell is x - 1
+    const int y0 = ((int)blockIdx.y * MAX3_WARPS + (int)threadIdx.y) * MAX3_ROWS;
+    const int z0 = (int)blockIdx.z * MAX3_PLANES;
+    const bool inx = x >= 1 && x <= nx;
+    const int put = threadIdx.x >= 1 && threadIdx.x <= 30 && x < gx ? min(MAX3_ROWS, gy - y0) : 0;
+    float a[MAX3_ROWS], b[MAX3_ROWS];  // 3 x 3 maxima of the last two planes
+#pragma unroll
+    for (int r = 0; r < MAX3_ROWS; ++r) a[r] = b[r] = 0.0f;
+    const float *src = in + ((long long)(z0 - 2) * ny + (y0 - 2)) * nx + (x - 1);  // read inside the grid only
+    float *dst = out + ((long long)z0 * gy + y0) * gx + x;
+#pragma unroll 2
+    for (int o = 0; o < MAX3_PLANES + 2; ++o, src += (long long)nx * ny) {
+        const int z = z0 - 2 + o;  // plane z of the grid, the last of three around plane z of the grown grid
+        const bool inz = inx && z >= 0 && z < nz;
+        float v[MAX3_ROWS + 2];
+#pragma unroll
+        for (int r = 0; r < MAX3_ROWS + 2; ++r) {  // rows y0 - 2 + r of the grid
+            const float w = inz && (unsigned)(y0 - 2 + r) < (unsigned)ny ? __ldg(src + (long long)r * nx) : 0.0f;
+            v[r] = w > 0.0f ? w : 0.0f;
+        }
+#pragma unroll
+        for (int r = 0; r < MAX3_ROWS; ++r) {
+            const float m = fmaxf(v[r], fmaxf(v[r + 1], v[r + 2]));
+            const float c = fmaxf(m, fmaxf(__shfl_up_sync(0xffffffffu, m, 1), __shfl_down_sync(0xffffffffu, m, 1)));
+            if (o >= 2 && z < gz && r < put) dst[(long long)r * gx] = fmaxf(c, fmaxf(a[r], b[r]));
+            a[r] = b[r];
+            b[r] = c;
+        }
+        if (o >= 2) dst += (long long)gx * gy;
+    }
+}
+
+// One pass of the separable maximum filter for wider neighbourhoods (a finite star): out = max
+// over the 2D + 1 values of `in` along axis `ax` around each cell of the grown grid
+// [nz + 2D][ny + 2D][nx + 2D].  In the first pass `in` is the grid itself (read at the offset
+// -D, zero outside it).
 __global__ void __launch_bounds__(256) k_max_filter(const float *__restrict__ in, float *__restrict__ out, int nx,
                                                     int ny, int nz, int D, int ax, int first)
 {
@@ -62,98 +105,124 @@ __global__ void __launch_bounds__(256) k_max_filter(const float *__restrict__ in
 }
 
 struct SkyGeom {
-    double lo[3], h[3];  // the grid proper
-    int n[3], D;
-    double hmin, R, tmax;  // smallest cell edge, start radius, longest path inside the grid
+    float lo[3], h[3];  // the grown box's lower corner, the cell edges
+    int n[3];           // cells of the grown box
+    float R, tmax, room;  // start radius, longest path inside the grid, R + t alpha stays below room
     int m;
 };
 
-// Direction of face f at face coordinates (u, v), not normalised.
-__device__ __forceinline__ void face_dir(int f, double u, double v, double d[3])
-{
-    const int a = f >> 1;
-    const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
-    d[a] = (f & 1) ? -1.0 : 1.0;
-    d[b] = u;
-    d[c] = v;
-}
-
-__global__ void __launch_bounds__(256) k_sky_walk(const float *__restrict__ K, SkyGeom g, double *map)
+// One walk per texel, in float: the set-up in double took most of the 0.79 ms of 6 x 320^2
+// texels on the 256^3 disk (FP64 runs at 1/64 of the float rate), and a walk that indexes its
+// axis state by the axis keeps it in local memory.  In float with the axes unrolled 381 us, in
+// patches of 8 x 4 texels a warp 297, with face parameters by one fused multiply-add and no cell
+// counters 200: issue-bound (76 % of the slots).  The geometry runs four cells ahead of the sum, so
+// four loads are in flight.
+constexpr int SKY_BATCH = 4;
+__global__ void __launch_bounds__(256) k_sky_walk(const float *__restrict__ K, const __grid_constant__ SkyGeom g,
+                                                  double *__restrict__ map)
 {
     const int m = g.m;
-    const long long texels = 6LL * m * m;
-    const double inf = __longlong_as_double(0x7ff0000000000000ll);
-    const int gn[3] = {g.n[0] + 2 * g.D, g.n[1] + 2 * g.D, g.n[2] + 2 * g.D};
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < texels;
-         t += (long long)gridDim.x * blockDim.x) {
-        const int f = (int)(t / ((long long)m * m)), iv = (int)((t / m) % m), iu = (int)(t % m);
-        const double du = 2.0 / m, u0 = -1.0 + iu * du, v0 = -1.0 + iv * du;
-        double u[3];
-        face_dir(f, u0 + 0.5 * du, v0 + 0.5 * du, u);
-        const double un = sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-        for (int a = 0; a < 3; ++a) u[a] /= un;
-        // the texel is a convex patch of the face: its directions lie within the largest
-        // angle between u and its corners
-        double cmin = 1.0;
+    const float inf = __int_as_float(0x7f800000);
+    // a warp takes patches of 8 x 4 texels: its rays stay closer together than along a row, where
+    // on two of the faces every ray reads its own row of the grid
+    const unsigned pu = (m + 7) / 8, pv = (m + 3) / 4, patches = 6 * pu * pv, lane = threadIdx.x & 31;
+    const unsigned warps = gridDim.x * (blockDim.x / 32);
+    for (unsigned p = (blockIdx.x * blockDim.x + threadIdx.x) / 32; p < patches; p += warps) {
+        const int f = (int)(p / (pu * pv)), q = (int)(p - f * (pu * pv));
+        const int iv = q / (int)pu * 4 + (int)(lane >> 3), iu = q % (int)pu * 8 + (int)(lane & 7);
+        if (iu >= m || iv >= m) continue;
+        const unsigned t = ((unsigned)f * m + iv) * m + iu;
+        const float du = 1.0f / m;  // half a texel
+        const float u = (2 * iu + 1) * du - 1.0f, v = (2 * iv + 1) * du - 1.0f;
+        // the texel is a convex patch of the face, so its directions lie within the largest
+        // angle between its centre (1, u, v) and its corners: sin = |centre x corner| / (|centre| |corner|)
+        const float c2 = 1.0f + u * u + v * v;
+        float s2 = 0.0f;
+#pragma unroll
         for (int k = 0; k < 4; ++k) {
-            double w[3];
-            face_dir(f, u0 + (k & 1) * du, v0 + (k >> 1) * du, w);
-            const double wn = sqrt(w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
-            cmin = fmin(cmin, (u[0] * w[0] + u[1] * w[1] + u[2] * w[2]) / wn);
+            const float eu = (k & 1) ? du : -du, ev = (k & 2) ? du : -du;
+            const float cu = u + eu, cv = v + ev, w = u * ev - v * eu;
+            s2 = fmaxf(s2, (w * w + eu * eu + ev * ev) / (c2 * (1.0f + cu * cu + cv * cv)));
         }
-        const double alpha = acos(fmax(fmin(cmin, 1.0), -1.0)) * (1.0 + 1e-6) + 1e-12;
-        // the walk below runs in float: its cell boundaries (face distances recomputed from
-        // the cell index at every step, never accumulated) sit within 1e-6 of the medium of
-        // the exact ones, taken off the room the neighbourhoods leave
-        if (g.R + g.tmax * alpha > g.D * g.hmin - 1e-6 * (1.0 + g.tmax)) {
-            map[t] = inf;
+        // (each angle is below 60 degrees; the margins cover the float rounding of the sine and
+        // of the centre's direction)
+        const float alpha = asinf(fminf(sqrtf(s2), 1.0f)) * (1.0f + 1e-5f) + 1e-6f;
+        if (!(g.R + g.tmax * alpha <= g.room)) {
+            map[t] = (double)inf;
             continue;
         }
-        // the centre ray from the origin through the grown box [blo, bhi]
-        double blo[3], bhi[3], t0 = 0.0, t1 = inf;
+        // the centre ray from the origin through the grown box
+        const float un = rsqrtf(c2), w = (f & 1) ? -un : un;
+        const int ax = f >> 1;
+        const float d[3] = {ax == 0 ? w : u * un, ax == 1 ? w : (ax == 0 ? u : v) * un, ax == 2 ? w : v * un};
+        float t0 = 0.0f, t1 = inf;
         bool miss = false;
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
-            blo[a] = g.lo[a] - g.D * g.h[a];
-            bhi[a] = g.lo[a] + (g.n[a] + g.D) * g.h[a];
-            if (u[a] != 0.0) {
-                double ta = blo[a] / u[a], tb = bhi[a] / u[a];
-                if (ta > tb) {
-                    const double x = ta;
-                    ta = tb;
-                    tb = x;
-                }
-                t0 = fmax(t0, ta);
-                t1 = fmin(t1, tb);
-            } else if (0.0 < blo[a] || 0.0 >= bhi[a]) {
+            const float lo = g.lo[a], hi = lo + g.n[a] * g.h[a];
+            if (d[a] != 0.0f) {
+                const float ta = lo / d[a], tb = hi / d[a];
+                t0 = fmaxf(t0, fminf(ta, tb));
+                t1 = fminf(t1, fmaxf(ta, tb));
+            } else if (0.0f < lo || 0.0f >= hi) {
                 miss = true;
             }
         }
+        t0 *= 1.0f - 1e-6f;  // a little early
         float sum = 0.0f;
         if (!miss && t1 > t0) {
-            int c[3], step[3];
-            float face0[3], hf[3], iu_[3], next[3];
+            // per axis: the first face's parameter and the spacing of the faces, faces crossed so
+            // far, the next face's parameter, the index step
+            float n0[3], dt[3], cnt[3] = {0.0f, 0.0f, 0.0f}, next[3], tend = inf;
+            unsigned st[3], off = 0, stride = 1;  // the tracer's grids hold at most 2^31 cells: indices modulo 2^32
+#pragma unroll
             for (int a = 0; a < 3; ++a) {
-                // a start on a face may pick the cell on either side: K_D of either bounds
-                // the other's cell (D >= 1), and a wrong side is left after a zero length
-                c[a] = min(max((int)floor((t0 * u[a] - blo[a]) / g.h[a]), 0), gn[a] - 1);
-                step[a] = u[a] > 0.0 ? 1 : u[a] < 0.0 ? -1 : 0;
-                face0[a] = (float)(blo[a] + (u[a] > 0.0 ? g.h[a] : 0.0));  // exit face of cell 0
-                hf[a] = (float)g.h[a];
-                iu_[a] = u[a] != 0.0 ? (float)(1.0 / u[a]) : 0.0f;
-                next[a] = step[a] ? (face0[a] + (float)c[a] * hf[a]) * iu_[a] : __int_as_float(0x7f800000);
+                // a start on a face may pick the cell on either side: the neighbourhood maximum of
+                // either bounds the other's cell, and a wrong side is left after a zero length
+                const int c = min(max((int)floorf((t0 * d[a] - g.lo[a]) / g.h[a]), 0), g.n[a] - 1);
+                const int left = d[a] > 0.0f ? g.n[a] - 1 - c : c;
+                n0[a] = next[a] = inf;
+                dt[a] = 0.0f;
+                if (d[a] != 0.0f) {
+                    n0[a] = next[a] = (g.lo[a] + (float)(d[a] > 0.0f ? c + 1 : c) * g.h[a]) / d[a];
+                    dt[a] = g.h[a] / fabsf(d[a]);
+                    // the face through which the axis leaves the box, as the walk will compute it:
+                    // no step is taken from tend on, so none leaves the box
+                    tend = fminf(tend, fmaf((float)left, dt[a], n0[a]));
+                }
+                st[a] = d[a] > 0.0f ? stride : 0u - stride;
+                off += (unsigned)c * stride;
+                stride *= (unsigned)g.n[a];
             }
-            float tc = (float)t0;
-            const float tend = (float)t1;
+            float tc = t0;
             while (tc < tend) {
-                int a = 0;
-                if (next[1] < next[a]) a = 1;
-                if (next[2] < next[a]) a = 2;
-                const float te = fminf(next[a], tend);
-                sum += K[((long long)c[2] * gn[1] + c[1]) * gn[0] + c[0]] * fmaxf(te - tc, 0.0f);
-                tc = fmaxf(tc, te);
-                c[a] += step[a];
-                if (c[a] < 0 || c[a] >= gn[a]) break;
-                next[a] = (face0[a] + (float)c[a] * hf[a]) * iu_[a];
+                float len[SKY_BATCH];
+                unsigned at[SKY_BATCH];
+#pragma unroll
+                for (int b = 0; b < SKY_BATCH; ++b) {
+                    const float tn = fminf(next[0], fminf(next[1], next[2])), te = fminf(tn, tend);
+                    at[b] = off;
+                    len[b] = fmaxf(te - tc, 0.0f);
+                    tc = fmaxf(tc, te);
+                    const bool go = tn < tend, x = go && next[0] == tn, y = go && !x && next[1] == tn, z = go && !x && !y;
+                    if (x) {  // face parameters from the crossing count, never accumulated
+                        off += st[0];
+                        cnt[0] += 1.0f;
+                        next[0] = fmaf(cnt[0], dt[0], n0[0]);
+                    }
+                    if (y) {
+                        off += st[1];
+                        cnt[1] += 1.0f;
+                        next[1] = fmaf(cnt[1], dt[1], n0[1]);
+                    }
+                    if (z) {
+                        off += st[2];
+                        cnt[2] += 1.0f;
+                        next[2] = fmaf(cnt[2], dt[2], n0[2]);
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < SKY_BATCH; ++b) sum += __ldg(K + at[b]) * len[b];
             }
         }
         // the cone ray and the centre ray cover equal lengths per t: the margin covers the
@@ -185,29 +254,45 @@ cudaError_t launch_sky_bound(const float *k, int nx, int ny, int nz, const doubl
     float *A = (float *)ws;
     float *B = (float *)((char *)ws + ((cells * 4 + 255) & ~255ull));
     const unsigned grid = (unsigned)std::min<uint64_t>((cells + 255) / 256, 152ull * 32);
-    k_max_filter<<<grid, 256, 0, s>>>(k, A, nx, ny, nz, D, 0, 1);
-    k_max_filter<<<grid, 256, 0, s>>>(A, B, nx, ny, nz, D, 1, 0);
-    k_max_filter<<<grid, 256, 0, s>>>(B, A, nx, ny, nz, D, 2, 0);
+    if (D == 1) {
+        const dim3 blocks((nx + 2 + 29) / 30, (ny + 2 + MAX3_ROWS * MAX3_WARPS - 1) / (MAX3_ROWS * MAX3_WARPS),
+                          (nz + 2 + MAX3_PLANES - 1) / MAX3_PLANES);
+        if (blocks.y <= 65535 && blocks.z <= 65535) {
+            k_max_filter3<<<blocks, dim3(32, MAX3_WARPS), 0, s>>>(k, A, nx, ny, nz);
+        } else {  // an axis of over half a million cells
+            k_max_filter<<<grid, 256, 0, s>>>(k, A, nx, ny, nz, D, 0, 1);
+            k_max_filter<<<grid, 256, 0, s>>>(A, B, nx, ny, nz, D, 1, 0);
+            k_max_filter<<<grid, 256, 0, s>>>(B, A, nx, ny, nz, D, 2, 0);
+        }
+    } else {
+        k_max_filter<<<grid, 256, 0, s>>>(k, A, nx, ny, nz, D, 0, 1);
+        k_max_filter<<<grid, 256, 0, s>>>(A, B, nx, ny, nz, D, 1, 0);
+        k_max_filter<<<grid, 256, 0, s>>>(B, A, nx, ny, nz, D, 2, 0);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     SkyGeom g;
-    g.D = D;
     g.m = m;
-    g.R = radius;
+    g.R = (float)(radius * (1.0 + 1e-6));
     const int n[3] = {nx, ny, nz};
-    g.hmin = 1e300;
-    double far2 = 0.0;
+    double hmin = 1e300, far2 = 0.0;
     for (int a = 0; a < 3; ++a) {
-        g.lo[a] = lo[a];
-        g.n[a] = n[a];
-        g.h[a] = (hi[a] - lo[a]) / n[a];
-        g.hmin = std::min(g.hmin, g.h[a]);
+        const double h = (hi[a] - lo[a]) / n[a];
+        g.lo[a] = (float)(lo[a] - D * h);
+        g.n[a] = n[a] + 2 * D;
+        g.h[a] = (float)h;
+        hmin = std::min(hmin, h);
         const double ext = std::max(std::fabs(lo[a]), std::fabs(hi[a])) + radius;
         far2 += ext * ext;
     }
-    g.tmax = std::sqrt(far2);  // from within R of the origin to the farthest point of the grid
-    const long long texels = 6LL * m * m;
-    const unsigned tgrid = (unsigned)std::min<long long>((texels + 255) / 256, 152LL * 32);
+    const double tmax = std::sqrt(far2);  // from within R of the origin to the farthest point of the grid
+    g.tmax = (float)(tmax * (1.0 + 1e-6));
+    // the walk's cell boundaries (face parameters recomputed from the cell index, never
+    // accumulated) sit within 2e-6 of the medium of the exact ones, taken off the room the
+    // neighbourhoods leave
+    g.room = (float)((D * hmin - 2e-6 * (1.0 + tmax)) * (1.0 - 1e-6));
+    const long long patches = 6LL * ((m + 7) / 8) * ((m + 3) / 4);
+    const unsigned tgrid = (unsigned)std::min<long long>((patches + 7) / 8, 152LL * 32);
     k_sky_walk<<<tgrid, 256, 0, s>>>(A, g, map);
     return cudaGetLastError();
 }

@@ -42,30 +42,115 @@ __device__ __forceinline__ long long block_index(const int nb[3], int x, int y, 
 }
 
 // K_b: the largest value of each block's cells (the padded grid holds +0 for empty cells
-// and -0 in the padding; neither raises the maximum).
-__global__ void __launch_bounds__(256) k_tail_block_max(const float *__restrict__ K, int nx, int ny, int nz, int pad,
+// and -0 in the padding; neither raises the maximum, so a block that reaches past the grid may
+// read its whole cube: pad >= TAIL_BLOCK).  VEC: rows of a block as one 16-byte vector.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_tail_block_max(const float *__restrict__ K, int nx, int ny, int pad,
                                                         TailGeom g, float *__restrict__ Kb)
 {
-    const long long px = nx + 2 * pad, py = ny + 2 * pad;
-    const long long blocks = (long long)g.nb[0] * g.nb[1] * g.nb[2];
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < blocks;
-         q += (long long)gridDim.x * blockDim.x) {
-        const int bx = (int)(q % g.nb[0]), by = (int)((q / g.nb[0]) % g.nb[1]),
-                  bz = (int)(q / ((long long)g.nb[0] * g.nb[1]));
+    const unsigned px = nx + 2 * pad, py = ny + 2 * pad;  // a padded grid holds at most 2^31 cells
+    const unsigned blocks = (unsigned)g.nb[0] * g.nb[1] * g.nb[2];
+    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < blocks; q += gridDim.x * blockDim.x) {
+        const unsigned w = q / g.nb[0], bx = q - w * g.nb[0], bz = w / g.nb[1], by = w - bz * g.nb[1];
+        const float *base = K + ((bz * TAIL_BLOCK + pad) * py + (by * TAIL_BLOCK + pad)) * px + (bx * TAIL_BLOCK + pad);
         float m = 0.0f;
-        for (int z = bz * TAIL_BLOCK; z < min(nz, (bz + 1) * TAIL_BLOCK); ++z)
-            for (int y = by * TAIL_BLOCK; y < min(ny, (by + 1) * TAIL_BLOCK); ++y)
-                for (int x = bx * TAIL_BLOCK; x < min(nx, (bx + 1) * TAIL_BLOCK); ++x) {
-                    const float v = __ldg(K + ((z + pad) * py + (y + pad)) * px + (x + pad));
-                    if (v > m) m = v;
+#pragma unroll
+        for (unsigned z = 0; z < TAIL_BLOCK; ++z)
+#pragma unroll
+            for (unsigned y = 0; y < TAIL_BLOCK; ++y) {
+                const float *row = base + (z * py + y) * px;
+                if (VEC) {
+                    const float4 v = __ldg(reinterpret_cast<const float4 *>(row));
+                    m = fmaxf(m, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                } else {
+#pragma unroll
+                    for (int x = 0; x < TAIL_BLOCK; ++x) m = fmaxf(m, __ldg(row + x));
                 }
+            }
         Kb[q] = m;
     }
 }
 
+// The lateral maxima of every slab, into the place of the slab's bounds: the part of the
+// recurrence that does not depend on the slab before.
+__global__ void __launch_bounds__(256) k_tail_lateral(const float *__restrict__ Kb, TailGeom g, float *__restrict__ Bb)
+{
+    const unsigned blocks = (unsigned)g.nb[0] * g.nb[1] * g.nb[2];
+    for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < blocks; q += gridDim.x * blockDim.x) {
+        const unsigned w = q / g.nb[0];
+        const int at[3] = {(int)(q - w * g.nb[0]), (int)(w % g.nb[1]), (int)(w / g.nb[1])};
+        const int ib = g.b == 0 ? at[0] : at[1], ic = g.c == 2 ? at[2] : at[1];
+        float m = 0.0f;
+        for (int ob = 0; ob < g.lb; ++ob) {
+            if ((unsigned)(ib + g.sb * ob) >= (unsigned)g.nbb) break;
+            for (int oc = 0; oc < g.lc; ++oc) {
+                if ((unsigned)(ic + g.sc * oc) >= (unsigned)g.nbc) break;
+                m = fmaxf(m, __ldg(Kb + (long long)q + g.sb * ob * g.tb + g.sc * oc * g.tc));
+            }
+        }
+        Bb[q] = m;
+    }
+}
+
 // The slab recurrence, one block of threads: slab after slab against the direction, every
-// block of a slab in parallel.
-__global__ void __launch_bounds__(1024) k_tail_slabs(const float *__restrict__ Kb, TailGeom g, float *__restrict__ Bb)
+// block of a slab in parallel.  The bounds of the slab before are kept in shared memory and
+// maximised along one lateral axis, then along the other, inside a margin of zeros that takes
+// the place of bounds checks; a thread's lateral maxima of the next slab are loaded before it
+// waits.  Serial over the slabs on one SM: at 64 slabs of 64 x 64 blocks 57 us (380 with nine
+// reads a block through L2, 105 with checked offsets).
+constexpr int SLAB_MARGIN = 2;  // lateral offsets reach 2 blocks either way
+__host__ __device__ constexpr int slab_words(int nbb, int nbc)
+{
+    return (nbb + 2 * SLAB_MARGIN) * (nbc + 2 * SLAB_MARGIN);
+}
+
+template <int PER>
+__global__ void __launch_bounds__(1024) k_tail_slabs(TailGeom g, float *__restrict__ Bb)
+{
+    extern __shared__ float s_slab[];  // bounds of the slab before, then their maxima along b
+    const int na = g.na, nbb = g.nbb, per_slab = g.nbb * g.nbc, pitch = nbb + 2 * SLAB_MARGIN;
+    float *B = s_slab, *M = s_slab + slab_words(nbb, g.nbc);
+    for (int t = threadIdx.x; t < 2 * slab_words(nbb, g.nbc); t += 1024) s_slab[t] = 0.0f;
+    // an axis the ray moves along by fewer blocks repeats an offset: the maximum is the same
+    const int b1 = g.lb > 1 ? g.sb : 0, b2 = g.lb > 2 ? 2 * g.sb : b1;
+    const int c1 = g.lc > 1 ? g.sc * pitch : 0, c2 = g.lc > 2 ? 2 * g.sc * pitch : c1;
+    int at[PER];      // index in the slab's array, 0 for no block
+    long long to[PER];  // index in Bb
+    float k[PER];
+    const long long down = g.sa > 0 ? -g.ta : g.ta;  // to the slab after this one
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+        const int t = threadIdx.x + p * 1024, ic = t / nbb, ib = t - ic * nbb;
+        at[p] = t < per_slab ? (ic + SLAB_MARGIN) * pitch + ib + SLAB_MARGIN : 0;
+        to[p] = (g.sa > 0 ? na - 1 : 0) * g.ta + ib * g.tb + ic * g.tc;  // the exit side first
+        k[p] = at[p] ? Bb[to[p]] : 0.0f;
+    }
+    __syncthreads();
+    for (int step = 0; step < na; ++step) {
+        float ahead[PER];
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            ahead[p] = at[p] && step + 1 < na ? Bb[to[p] + down] : 0.0f;
+            if (at[p]) M[at[p]] = fmaxf(B[at[p]], fmaxf(B[at[p] + b1], B[at[p] + b2]));
+        }
+        __syncthreads();
+#pragma unroll
+        for (int p = 0; p < PER; ++p) {
+            if (at[p]) {
+                const float m = fmaxf(M[at[p]], fmaxf(M[at[p] + c1], M[at[p] + c2]));
+                const float b = __fadd_ru(__fmul_ru(k[p], g.path), m);
+                B[at[p]] = b;
+                Bb[to[p]] = b;
+            }
+            to[p] += down;
+            k[p] = ahead[p];
+        }
+        __syncthreads();
+    }
+}
+
+// The same recurrence through global memory, for slabs too large for shared memory.
+__global__ void __launch_bounds__(1024) k_tail_slabs_wide(TailGeom g, float *__restrict__ Bb)
 {
     const int na = g.na, nbb = g.nbb, nbc = g.nbc;
     const int per_slab = nbb * nbc;
@@ -74,47 +159,76 @@ __global__ void __launch_bounds__(1024) k_tail_slabs(const float *__restrict__ K
         const int jn = j + g.sa;                          // the slab a ray from slab j enters next
         for (int t = threadIdx.x; t < per_slab; t += blockDim.x) {
             const int ib = t % nbb, ic = t / nbb;
-            float kmax = 0.0f, nmax = 0.0f;
-            for (int ob = 0; ob < g.lb; ++ob) {
+            float nmax = 0.0f;
+            for (int ob = 0; step && ob < g.lb; ++ob) {
                 const int qb = ib + g.sb * ob;
                 if (qb < 0 || qb >= nbb) continue;
                 for (int oc = 0; oc < g.lc; ++oc) {
                     const int qc = ic + g.sc * oc;
                     if (qc < 0 || qc >= nbc) continue;
-                    const long long lat = qb * g.tb + qc * g.tc;
-                    kmax = fmaxf(kmax, Kb[j * g.ta + lat]);
-                    if (jn >= 0 && jn < na) nmax = fmaxf(nmax, Bb[jn * g.ta + lat]);
+                    nmax = fmaxf(nmax, Bb[jn * g.ta + qb * g.tb + qc * g.tc]);
                 }
             }
-            Bb[j * g.ta + ib * g.tb + ic * g.tc] = __fadd_ru(__fmul_ru(kmax, g.path), nmax);
+            float *b = Bb + j * g.ta + ib * g.tb + ic * g.tc;
+            *b = __fadd_ru(__fmul_ru(*b, g.path), nmax);
         }
         __syncthreads();
     }
 }
 
-// Codes of the padded grid's cells: c = (biased exponent of B, at least 1) + 24, so that
-// B < 2^(c - 150); 0 for B = 0 and for the padding; 255 above 2^104 or not finite.
+// Code of a bound: c = (biased exponent of B, at least 1) + 24, so that B < 2^(c - 150); 0 for
+// B = 0; 255 above 2^104 or not finite.
+__device__ __forceinline__ uint32_t tail_code(float B)
+{
+    if (!(B <= 3.0e38f)) return 255u;
+    if (!(B > 0.0f)) return 0u;
+    const int E = (int)((__float_as_uint(B) >> 23) & 0xffu);
+    const int c = max(E, 1) + 24;
+    return c > 254 ? 255u : (uint32_t)c;
+}
+
+// Codes of the padded grid's cells (0 in the padding), a warp per row: the row's blocks are
+// found once, and VEC writes the four cells of a block, which share its code, as one word
+// (rows and padding of whole blocks).  16 us at 256^3 (79 with divisions and a
+// byte store a cell).
+template <bool VEC>
 __global__ void __launch_bounds__(256) k_tail_expand(const float *__restrict__ Bb, int nx, int ny, int nz, int pad,
                                                      TailGeom g, uint8_t *__restrict__ map)
 {
-    const long long px = nx + 2 * pad, py = ny + 2 * pad, pz = nz + 2 * pad;
-    const long long cells = px * py * pz;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < cells;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(e % px) - pad, y = (int)((e / px) % py) - pad, z = (int)(e / (px * py)) - pad;
-        uint8_t code = 0;
-        if (x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz) {
-            const float B = Bb[block_index(g.nb, x / TAIL_BLOCK, y / TAIL_BLOCK, z / TAIL_BLOCK)];
-            if (!(B <= 3.0e38f)) {
-                code = 255;
-            } else if (B > 0.0f) {
-                const int E = (int)((__float_as_uint(B) >> 23) & 0xffu);
-                const int c = max(E, 1) + 24;
-                code = (uint8_t)(c > 254 ? 255 : c);
+    const int px = nx + 2 * pad, py = ny + 2 * pad, pz = nz + 2 * pad;
+    const long long rows = (long long)py * pz;
+    const int lane = threadIdx.x & 31;
+    for (long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * 8) {
+        const int z = (int)(r / py) - pad, y = (int)(r % py) - pad;
+        const bool in = z >= 0 && z < nz && y >= 0 && y < ny;
+        const float *src = Bb + block_index(g.nb, 0, in ? y / TAIL_BLOCK : 0, in ? z / TAIL_BLOCK : 0);
+        uint8_t *dst = map + r * px;
+        if (VEC) {
+            for (int v = lane; v < px / 4; v += 32) {
+                const int x = 4 * v - pad;
+                const uint32_t code = in && x >= 0 && x < nx ? tail_code(__ldg(src + x / TAIL_BLOCK)) : 0u;
+                reinterpret_cast<uint32_t *>(dst)[v] = code * 0x01010101u;
+            }
+        } else {
+            for (int c = lane; c < px; c += 32) {
+                const int x = c - pad;
+                dst[c] = (uint8_t)(in && x >= 0 && x < nx ? tail_code(__ldg(src + x / TAIL_BLOCK)) : 0u);
             }
         }
-        map[e] = code;
     }
+}
+
+template <int PER>
+cudaError_t launch_slabs(const TailGeom &g, float *Bb, cudaStream_t s)
+{
+    const size_t smem = 2 * sizeof(float) * (size_t)slab_words(g.nbb, g.nbc);
+    if (smem > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_tail_slabs<PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    k_tail_slabs<PER><<<1, 1024, smem, s>>>(g, Bb);
+    return cudaGetLastError();
 }
 
 int blocks_of(int n) { return (n + TAIL_BLOCK - 1) / TAIL_BLOCK; }
@@ -170,11 +284,27 @@ cudaError_t launch_tail_map(const float *k_padded, int nx, int ny, int nz, int p
     const uint64_t blocks = (uint64_t)g.nb[0] * g.nb[1] * g.nb[2];
     float *Bb = (float *)((char *)ws + aligned(blocks * sizeof(float)));
     const unsigned bgrid = (unsigned)std::min<uint64_t>((blocks + 255) / 256, 152ull * 16);
-    k_tail_block_max<<<bgrid, 256, 0, s>>>(k_padded, nx, ny, nz, pad, g, Kb);
-    k_tail_slabs<<<1, 1024, 0, s>>>(Kb, g, Bb);
-    const uint64_t cells = (uint64_t)(nx + 2 * pad) * (ny + 2 * pad) * (nz + 2 * pad);
-    const unsigned egrid = (unsigned)std::min<uint64_t>((cells + 255) / 256, 152ull * 32);
-    k_tail_expand<<<egrid, 256, 0, s>>>(Bb, nx, ny, nz, pad, g, map);
+    // whole vectors: a row of the padded grid, its padding and every block start on one
+    const bool whole = nx % TAIL_BLOCK == 0 && pad % TAIL_BLOCK == 0;
+    if (whole && ((uintptr_t)k_padded & 15) == 0) k_tail_block_max<true><<<bgrid, 256, 0, s>>>(k_padded, nx, ny, pad, g, Kb);
+    else k_tail_block_max<false><<<bgrid, 256, 0, s>>>(k_padded, nx, ny, pad, g, Kb);
+    k_tail_lateral<<<bgrid, 256, 0, s>>>(Kb, g, Bb);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const long long per_slab = (long long)g.nbb * g.nbc;
+    // a slab of up to 16 blocks a thread whose margins fit shared memory (128 x 128 blocks, a
+    // 512^3 grid, take 136 KB)
+    if (per_slab > 16 * 1024 || 8ull * (g.nbb + 2 * SLAB_MARGIN) * (g.nbc + 2 * SLAB_MARGIN) > 200 * 1024)
+        k_tail_slabs_wide<<<1, 1024, 0, s>>>(g, Bb);
+    else if (per_slab <= 1024) e = launch_slabs<1>(g, Bb, s);
+    else if (per_slab <= 4 * 1024) e = launch_slabs<4>(g, Bb, s);
+    else e = launch_slabs<16>(g, Bb, s);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const uint64_t rows = (uint64_t)(ny + 2 * pad) * (nz + 2 * pad);
+    const unsigned egrid = (unsigned)std::min<uint64_t>((rows + 7) / 8, 152ull * 16);
+    if (whole && ((uintptr_t)map & 3) == 0) k_tail_expand<true><<<egrid, 256, 0, s>>>(Bb, nx, ny, nz, pad, g, map);
+    else k_tail_expand<false><<<egrid, 256, 0, s>>>(Bb, nx, ny, nz, pad, g, map);
     return cudaGetLastError();
 }
 
