@@ -44,6 +44,10 @@ struct Mth<float> {
     static __device__ __forceinline__ float floor_(float x) { return floorf(x); }
     static __device__ __forceinline__ float min_(float a, float b) { return fminf(a, b); }
     static __device__ __forceinline__ float max_(float a, float b) { return fmaxf(a, b); }
+    // face distances of a walk: never negative, never -0 or NaN
+    static __device__ __forceinline__ float nearer(float a, float b) { return fminf(a, b); }
+    static __device__ __forceinline__ bool reached(float s) { return s == 0.0f; }
+    static __device__ __forceinline__ float cell(float k) { return k; }  // a density, or the sentinel -0
     static __device__ __forceinline__ float inf() { return __int_as_float(0x7f800000); }
     // value of a 32-bit point coordinate: x * 2^-32 rounded toward zero
     static __device__ __forceinline__ float from_u32(uint32_t x) { return __uint2float_rz(x) * 0x1p-32f; }
@@ -73,6 +77,23 @@ struct Mth<double> {
     static __device__ __forceinline__ double floor_(double x) { return floor(x); }
     static __device__ __forceinline__ double min_(double a, double b) { return fmin(a, b); }
     static __device__ __forceinline__ double max_(double a, double b) { return fmax(a, b); }
+    // Face distances of a walk are never negative, -0 or NaN, so their bits order as integers:
+    // the minima and the zero test of every cell, and the widening of its density, stay off
+    // the FP64 pipe (1/64 of the float rate), which keeps three subtractions and a fused
+    // multiply-add a cell of about nine operations.  200 000 Halton packets of a finite star,
+    // 64^3 disk: 1202 -> 866 us.
+    static __device__ __forceinline__ double nearer(double a, double b)
+    {
+        const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+        return __longlong_as_double(x < y ? x : y);
+    }
+    static __device__ __forceinline__ bool reached(double s) { return __double_as_longlong(s) == 0; }
+    static __device__ __forceinline__ double cell(float k)
+    {
+        const uint32_t b = __float_as_uint(k) & 0x7fffffffu;  // -0 (a sentinel) adds nothing, like +0
+        if (b - 1u < 0x007fffffu || b >= 0x7f800000u) return (double)k;  // subnormal, infinite
+        return __hiloint2double(b ? (int)((b >> 3) + 0x38000000u) : 0, (int)(b << 29));
+    }
     static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
     static __device__ __forceinline__ double from_u32(uint32_t x) { return (double)x * 0x1p-32; }
     static __device__ __forceinline__ double from_f64(double v) { return v; }
@@ -610,15 +631,15 @@ __device__ __forceinline__ unsigned padded_batch(const float *__restrict__ K, Pa
 #pragma unroll
     for (int u = 0; u < WALK_UNROLL; ++u) {
         cell[u] = R.idx;
-        const T l = Mth<T>::min_(R.X.s, Mth<T>::min_(R.Y.s, R.Z.s));
+        const T l = Mth<T>::nearer(R.X.s, Mth<T>::nearer(R.Y.s, R.Z.s));
         L[u] = l;
         R.X.s -= l;  // exact (zero) for the axis whose face is reached
         R.Y.s -= l;
         R.Z.s -= l;
-        if (R.X.s == T(0)) {  // ties step x, then y, then z
+        if (Mth<T>::reached(R.X.s)) {  // ties step x, then y, then z
             R.idx += R.X.step;
             R.X.s = R.X.dt;
-        } else if (R.Y.s == T(0)) {
+        } else if (Mth<T>::reached(R.Y.s)) {
             R.idx += R.Y.step;
             R.Y.s = R.Y.dt;
         } else {
@@ -646,7 +667,7 @@ __device__ __forceinline__ T padded_depth(const float *__restrict__ K, PaddedRay
         const unsigned sign = padded_batch(K, R, L, kf);
         T Bs = T(0);  // the batch's optical depth, one fused multiply-add per cell
 #pragma unroll
-        for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], (T)kf[u], Bs);
+        for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], Mth<T>::cell(kf[u]), Bs);
         const T y = Bs - comp;  // acc += Bs, compensated
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
@@ -672,7 +693,7 @@ __device__ __forceinline__ T padded_depth_tail(const float *__restrict__ K, Padd
         const unsigned sign = padded_batch(K, R, L, kf);
         T Bs = T(0);
 #pragma unroll
-        for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], (T)kf[u], Bs);
+        for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], Mth<T>::cell(kf[u]), Bs);
         const T y = Bs - comp;
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
@@ -714,7 +735,7 @@ __device__ __forceinline__ T padded_depth_marks(const float *__restrict__ K, Pad
         const unsigned sign = padded_batch(K, R, L, kf);
         T Bs = T(0);
 #pragma unroll
-        for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], (T)kf[u], Bs);
+        for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], Mth<T>::cell(kf[u]), Bs);
         const T y = Bs - comp;
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
@@ -750,7 +771,7 @@ __device__ __forceinline__ bool padded_march(const float *__restrict__ K, Padded
         T Bs = T(0);
 #pragma unroll
         for (int u = 0; u < WALK_UNROLL; ++u) {
-            dtau[u] = Mth<T>::mul_(L[u], (T)kf[u]);
+            dtau[u] = Mth<T>::mul_(L[u], Mth<T>::cell(kf[u]));
             Bs = Mth<T>::add_(Bs, dtau[u]);
         }
         T rem = acc - comp;
