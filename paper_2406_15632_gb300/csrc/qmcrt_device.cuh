@@ -656,11 +656,49 @@ __device__ __forceinline__ unsigned padded_batch(const float *__restrict__ K, Pa
     return sign;
 }
 
-// Raw optical depth from the state R to the edge of the grid.
+// Batches after which a walk from p along d has left the support of the medium (every later
+// cell is empty): where the ray leaves the ball and the cylinder of G.support, in cells crossed
+// until there, both with room for rounding; 0 if it never enters them.  The depth sum's value is
+// the same bit for bit: an empty batch adds +0 to the compensated total, which keeps the exact
+// value of acc - comp.  The corners of the box around a spherical envelope are a fifth of a
+// walk, where rays have spread the most: the 20-order clumpy envelope takes 17.9 ms with it
+// against 20.4 per 2^22 packets, 5.28 against 6.03 per 2^20; on a 32^3 grid there is
+// nothing to gain (5.29 against 5.26 per 2^20).
 template <class T>
-__device__ __forceinline__ T padded_depth(const float *__restrict__ K, PaddedRay<T> &R)
+__device__ __forceinline__ unsigned support_batches(const MediumP<T> &G, const T p[3], const T d[3],
+                                                    const PaddedRay<T> &R)
+{
+    const float ball = __ldg(G.support) + 2e-5f, cyl = __ldg(G.support + 1) + 2e-5f;  // float rounding of q and e
+    float q[3], e[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        q[a] = ((float)p[a] - G.mid[a]) * G.inv_half[a];
+        e[a] = (float)d[a] * G.inv_half[a];
+    }
+    // far root of |q + t e|^2 = r^2; a ray that misses, or leaves behind its start, has none ahead
+    auto leaves = [](float A, float B, float C) {
+        const float disc = B * B - A * C;
+        if (A == 0.0f) return C > 0.0f ? 0.0f : __int_as_float(0x7f800000);
+        return disc > 0.0f ? fmaxf((sqrtf(disc) - B) / A, 0.0f) : 0.0f;
+    };
+    const float A2 = e[0] * e[0] + e[1] * e[1], B2 = q[0] * e[0] + q[1] * e[1], C2 = q[0] * q[0] + q[1] * q[1];
+    float t = leaves(A2 + e[2] * e[2], B2 + q[2] * e[2], C2 + q[2] * q[2] - ball);
+    if (cyl < 2.0f) t = fminf(t, leaves(A2, B2, C2 - cyl));
+    if (t == 0.0f) return 0u;
+    // faces crossed per axis until t, one more each for the crossing at hand, and one for rounding
+    float cells = 2.0f;
+    cells += fmaxf((t - (float)R.X.s) * fabsf((float)d[0] * (float)G.inv_h[0]) + 1.0f, 0.0f);
+    cells += fmaxf((t - (float)R.Y.s) * fabsf((float)d[1] * (float)G.inv_h[1]) + 1.0f, 0.0f);
+    cells += fmaxf((t - (float)R.Z.s) * fabsf((float)d[2] * (float)G.inv_h[2]) + 1.0f, 0.0f);
+    return __float2uint_ru(cells * (1.0f / WALK_UNROLL));
+}
+
+// Raw optical depth from the state R to the edge of the grid; with CUT, over n_max batches.
+template <class T, bool CUT = false>
+__device__ __forceinline__ T padded_depth(const float *__restrict__ K, PaddedRay<T> &R, unsigned n_max = 0)
 {
     T acc = T(0), comp = T(0);
+    if (CUT && n_max == 0) return acc;
     for (;;) {
         T L[WALK_UNROLL];
         float kf[WALK_UNROLL];
@@ -672,7 +710,7 @@ __device__ __forceinline__ T padded_depth(const float *__restrict__ K, PaddedRay
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
         acc = s2;
-        if (sign & 0x80000000u) break;
+        if ((sign & 0x80000000u) || (CUT && --n_max == 0)) break;
     }
     return acc - comp;
 }
@@ -720,15 +758,16 @@ __device__ __forceinline__ T padded_depth_tail(const float *__restrict__ K, Padd
 // 2, 4, 8 and 16 batches (the finite star and the batch gain most from 8 to 16).
 constexpr unsigned MARK_GAP = 8;
 
-template <class T>
+template <class T, bool CUT>
 __device__ __forceinline__ T padded_depth_marks(const float *__restrict__ K, PaddedRay<T> &R, T w, T kscale,
-                                                WalkMark<T> mk[2], int &ia, bool &has_b)
+                                                WalkMark<T> mk[2], int &ia, bool &has_b, unsigned n_max)
 {
     T acc = T(0), comp = T(0), thr = T(0);
     unsigned nb = 0;  // batches walked: promotions are considered at every MARK_GAP-th
     ia = 0;
     has_b = false;
     mark_at(mk[0], R, T(0));
+    if (CUT && n_max == 0) return acc;
     for (;;) {
         T L[WALK_UNROLL];
         float kf[WALK_UNROLL];
@@ -740,7 +779,7 @@ __device__ __forceinline__ T padded_depth_marks(const float *__restrict__ K, Pad
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
         acc = s2;
-        if (sign & 0x80000000u) break;
+        if ((sign & 0x80000000u) || (CUT && nb + 1 == n_max)) break;
         if (++nb % MARK_GAP == 0 && acc >= thr) {  // the same batches in every lane of a warp
             if (has_b) ia ^= 1;  // A = B
             const T b = acc - comp;
@@ -866,13 +905,18 @@ __device__ __forceinline__ T tau_to_edge(const MediumP<T> &G, const T p[3], cons
 
 // Optical depth from p toward observer O (the peel-off walk), ended early by O's tail map
 // where the observer has one.
-template <class T>
+template <class T, bool CUT>
 __device__ __forceinline__ T tau_toward(const MediumP<T> &G, const ObsP<T> &O, const T p[3])
 {
     if (O.tail && G.kind == QMCRT_MEDIUM_GRID && G.pad) {
         PaddedRay<T> R;
         if (!padded_start(G, p, O.k, O.inv_k, R)) return T(0);
         return Mth<T>::mul_(padded_depth_tail(G.k, R, O.tail, O.tail_thr), G.kscale);
+    }
+    if (CUT && G.support) {
+        PaddedRay<T> R;
+        if (!padded_start(G, p, O.k, O.inv_k, R)) return T(0);
+        return Mth<T>::mul_(padded_depth<T, true>(G.k, R, support_batches(G, p, O.k, R)), G.kscale);
     }
     return tau_to_edge(G, p, O.k, O.inv_k);
 }
@@ -943,7 +987,7 @@ __device__ __forceinline__ double sky_bound(const MediumP<T> &G, const T d[3])
 // A ray from within the bound map's radius whose direction's bound (qmcrt_sky_bound, with
 // a factor of two for the float walk's rounding) lies below tau_min cannot reach it: the
 // packet is skipped as the walk would skip it, without walking.
-template <class T>
+template <class T, bool CUT = false>
 __device__ __forceinline__ bool forced_step(const TraceP<T> &P, T pos[3], const T d[3], T w, T &W1)
 {
     if (P.med.sky && dot3(pos, pos) <= P.med.sky_r2 &&
@@ -967,7 +1011,9 @@ __device__ __forceinline__ bool forced_step(const TraceP<T> &P, T pos[3], const 
     WalkMark<T> mk[2];
     int ia;
     bool has_b;
-    const T raw1 = padded_depth_marks(P.med.k, R, w, P.med.kscale, mk, ia, has_b);
+    unsigned n_max = 0xffffffffu;
+    if (CUT && P.med.support) n_max = support_batches(P.med, pos, d, R);
+    const T raw1 = padded_depth_marks<T, CUT>(P.med.k, R, w, P.med.kscale, mk, ia, has_b, n_max);
     const T tau1 = Mth<T>::mul_(raw1, P.med.kscale);
     if (!(tau1 >= P.tau_min)) return false;
     W1 = -Mth<T>::expm1_(-tau1);
@@ -1154,7 +1200,7 @@ __device__ __forceinline__ bool peel_unpolarized(const TraceP<T> &P, const ObsP<
     x = dot3(pos, O.ex);
     y = dot3(pos, O.ey);
     if (occulted(P, O, pos)) return false;
-    const T tau_obs = tau_toward(P.med, O, pos);
+    const T tau_obs = tau_toward<T, false>(P.med, O, pos);
     const T mu = dot3(d, O.k);
     const T f = W0 * Mth<T>::exp_(-tau_obs) * hg_p11(P.dust, mu) * T(0.07957747154594767);  // 1/(4 pi)
     const T dx = dot3(d, O.ex), dy = dot3(d, O.ey);
@@ -1166,14 +1212,14 @@ __device__ __forceinline__ bool peel_unpolarized(const TraceP<T> &P, const ObsP<
 }
 
 // Peel-off of a polarized packet (direction n, Stokes S in the frame of axis a).
-template <class T>
+template <class T, bool CUT = false>
 __device__ __forceinline__ bool peel_polarized(const TraceP<T> &P, const ObsP<T> &O, const T pos[3], const T n[3],
                                                const T a[3], const T S[3], T out[3], T &x, T &y)
 {
     x = dot3(pos, O.ex);
     y = dot3(pos, O.ey);
     if (occulted(P, O, pos)) return false;
-    const T tau_obs = tau_toward(P.med, O, pos);
+    const T tau_obs = tau_toward<T, CUT>(P.med, O, pos);
     const T mu = dot3(n, O.k);
     const T inv1pm2 = T(1) / (T(1) + mu * mu);
     const T r12 = -P.dust.p_l * (T(1) - mu * mu) * inv1pm2;
@@ -1210,11 +1256,11 @@ __device__ __forceinline__ bool peel_unpolarized(const TraceP<T> &P, const T pos
     return peel_unpolarized(P, P.obs, pos, d, W0, S, x, y);
 }
 
-template <class T>
+template <class T, bool CUT = false>
 __device__ __forceinline__ bool peel_polarized(const TraceP<T> &P, const T pos[3], const T n[3], const T a[3],
                                                const T S[3], T out[3], T &x, T &y)
 {
-    return peel_polarized(P, P.obs, pos, n, a, S, out, x, y);
+    return peel_polarized<T, CUT>(P, P.obs, pos, n, a, S, out, x, y);
 }
 
 // HG scattering of a polarized packet (Sec. 3.5): Theta from v, azimuth 2 pi u from

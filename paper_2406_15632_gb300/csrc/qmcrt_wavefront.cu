@@ -63,7 +63,7 @@ static_assert(sizeof(Rec<float>) == 64 && sizeof(Rec<double>) == 128, "record si
 struct WaveCount {
     uint32_t live, chunk, space, pad;
 };
-static_assert(66 * sizeof(WaveCount) <= WV_TAIL_BYTES, "counters of every order (at most 64) and one more");
+static_assert(67 * sizeof(WaveCount) <= WV_TAIL_BYTES, "counters of every order (at most 64) and one more, the support");
 
 template <class T>
 struct WaveWork {
@@ -166,7 +166,7 @@ __device__ __forceinline__ bool run_order(const TraceP<T> &P, int k, uint64_t i,
     if (alive) {
         if (k == 1 || P.force_all) {
             T W1;
-            if (forced_step(P, p.pos, p.n, wd, W1)) {
+            if (forced_step<T, true>(P, p.pos, p.n, wd, W1)) {
                 p.S[0] *= W1;
                 p.S[1] *= W1;
                 p.S[2] *= W1;
@@ -184,7 +184,7 @@ __device__ __forceinline__ bool run_order(const TraceP<T> &P, int k, uint64_t i,
     }
     T out[3] = {T(0), T(0), T(0)};
     T x = T(0), y = T(0);
-    const bool contrib = alive && peel_polarized(P, p.pos, p.n, p.a, p.S, out, x, y);
+    const bool contrib = alive && peel_polarized<T, true>(P, p.pos, p.n, p.a, p.S, out, x, y);
     if (contrib && x >= -P.obs.hw && x < P.obs.hw && y >= -P.obs.hw && y < P.obs.hw) {
         p.tot += out[0];
         p.tot2 += out[0] * out[0];
@@ -354,6 +354,38 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) k_wave_order(cons
     }
 }
 
+// Support of a padded grid: the largest squared distance, in half edges of the box, of a nonzero
+// cell's farthest corner from the box centre (ball) and from the line along z through it
+// (cylinder).  One read of the grid a run.
+template <class T>
+__global__ void __launch_bounds__(256) k_wave_support(const __grid_constant__ MediumP<T> G, uint32_t *support)
+{
+    const int lane = threadIdx.x & 31, rows = G.n[1] * G.n[2], warps = gridDim.x * 8;
+    auto far2 = [](int c, int n) {
+        const float a = 2.0f * c / n - 1.0f, b = 2.0f * (c + 1) / n - 1.0f;
+        return fmaxf(a * a, b * b);
+    };
+    float ball = 0.0f, cyl = 0.0f;
+    for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += warps) {
+        const int z = r / G.n[1], y = r - z * G.n[1];
+        const float *row = G.k + ((size_t)(z + G.pad) * G.stride[2] + (size_t)(y + G.pad) * G.stride[1] + G.pad);
+        float x2 = -1.0f;
+        for (int x = lane; x < G.n[0]; x += 32)
+            if (__ldg(row + x) > 0.0f) x2 = fmaxf(x2, far2(x, G.n[0]));
+        if (x2 >= 0.0f) {
+            const float y2 = far2(y, G.n[1]);
+            cyl = fmaxf(cyl, x2 + y2);
+            ball = fmaxf(ball, x2 + y2 + far2(z, G.n[2]));
+        }
+    }
+    // positive floats order as integers
+    const uint32_t b = __reduce_max_sync(FULL_MASK, __float_as_uint(ball)), c = __reduce_max_sync(FULL_MASK, __float_as_uint(cyl));
+    if (lane == 0 && b) {
+        atomicMax(support, b);
+        atomicMax(support + 1, c);
+    }
+}
+
 template <class T>
 WaveWork<T> carve(void *ws, uint64_t cap)
 {
@@ -388,7 +420,7 @@ WaveKey wave_bits(uint64_t n, uint64_t queue_bytes)
 }
 
 template <class T>
-cudaError_t launch_wave(const TraceP<T> &P, void *ws, uint64_t cap, int sms, cudaStream_t s)
+cudaError_t launch_wave(TraceP<T> P, void *ws, uint64_t cap, int sms, cudaStream_t s)
 {
     if (P.count == 0) return cudaSuccess;
     WaveWork<T> W = carve<T>(ws, cap);
@@ -397,6 +429,11 @@ cudaError_t launch_wave(const TraceP<T> &P, void *ws, uint64_t cap, int sms, cud
     cudaError_t e = cudaMemsetAsync(W.count, 0, WV_TAIL_BYTES, s);
     if (e == cudaSuccess && P.max_orders > 1) e = cudaMemsetAsync(W.hist, 0, (size_t)buckets * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
+    if (P.med.kind == QMCRT_MEDIUM_GRID && P.med.pad) {
+        uint32_t *support = (uint32_t *)(W.count + 66);
+        k_wave_support<T><<<(unsigned)std::max(1, sms * 8), 256, 0, s>>>(P.med, support);
+        P.med.support = (const float *)support;
+    }
     const uint64_t threads = (P.ord.threads + 31) & ~31ull;
     k_wave_first<T><<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(P, W);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
