@@ -181,6 +181,11 @@ int batch_occupancy(int block, int precision);
 // Forward pass of the learned warp, both conditionals fused on the tensor cores.
 cudaError_t launch_warp_forward_fused(const float *params, const __nv_bfloat16 *wb, const float *u, float *x,
                                       float *logj, long long n, float mix, int *error, cudaStream_t s);
+// Loss and gradient of the learned warp on n logged samples, summed pass by pass of pass_rows rows
+// (a multiple of 128); sums: scratch of 33 doubles.
+cudaError_t launch_warp_train(const float *params, const __nv_bfloat16 *wb, const float *x, const float *w, long long n,
+                              long long pass_rows, float mix, float *grad, float *loss, double *sums, int *error,
+                              cudaStream_t s);
 cudaError_t launch_generate_points(const PointsP &p, uint64_t first, uint64_t count, int format, void *out,
                                    cudaStream_t s);
 cudaError_t launch_pad_grid(const float *k, int nx, int ny, int nz, int pad, float *out, cudaStream_t s);
