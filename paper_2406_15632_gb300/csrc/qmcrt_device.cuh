@@ -622,9 +622,11 @@ __device__ __forceinline__ bool padded_start(const MediumP<T> &G, const T p[3], 
 }
 
 // One batch: the segment lengths and cell values of the next WALK_UNROLL cells; returns
-// the OR of the values' bits (sign bit set: the ray has left the grid).
+// whether the ray has left the grid, which the last cell's sign tells: a ray that leaves
+// within the batch stays outside, in the padding (the four signs together cost 2 % on the disk:
+// 11.30 -> 11.09 ms per 2^26 packets).
 template <class T>
-__device__ __forceinline__ unsigned padded_batch(const float *__restrict__ K, PaddedRay<T> &R, T L[WALK_UNROLL],
+__device__ __forceinline__ bool padded_batch(const float *__restrict__ K, PaddedRay<T> &R, T L[WALK_UNROLL],
                                                  float kf[WALK_UNROLL])
 {
     unsigned cell[WALK_UNROLL];
@@ -647,13 +649,9 @@ __device__ __forceinline__ unsigned padded_batch(const float *__restrict__ K, Pa
             R.Z.s = R.Z.dt;
         }
     }
-    unsigned sign = 0u;
 #pragma unroll
-    for (int u = 0; u < WALK_UNROLL; ++u) {
-        kf[u] = __ldg(K + cell[u]);
-        sign |= __float_as_uint(kf[u]);
-    }
-    return sign;
+    for (int u = 0; u < WALK_UNROLL; ++u) kf[u] = __ldg(K + cell[u]);
+    return __float_as_int(kf[WALK_UNROLL - 1]) < 0;
 }
 
 // Batches after which a walk from p along d has left the support of the medium (every later
@@ -702,7 +700,7 @@ __device__ __forceinline__ T padded_depth(const float *__restrict__ K, PaddedRay
     for (;;) {
         T L[WALK_UNROLL];
         float kf[WALK_UNROLL];
-        const unsigned sign = padded_batch(K, R, L, kf);
+        const bool left = padded_batch(K, R, L, kf);
         T Bs = T(0);  // the batch's optical depth, one fused multiply-add per cell
 #pragma unroll
         for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], Mth<T>::cell(kf[u]), Bs);
@@ -710,7 +708,7 @@ __device__ __forceinline__ T padded_depth(const float *__restrict__ K, PaddedRay
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
         acc = s2;
-        if ((sign & 0x80000000u) || (CUT && --n_max == 0)) break;
+        if (left || (CUT && --n_max == 0)) break;
     }
     return acc - comp;
 }
@@ -728,7 +726,7 @@ __device__ __forceinline__ T padded_depth_tail(const float *__restrict__ K, Padd
         const int code = __ldg(tail + R.idx);
         T L[WALK_UNROLL];
         float kf[WALK_UNROLL];
-        const unsigned sign = padded_batch(K, R, L, kf);
+        const bool left = padded_batch(K, R, L, kf);
         T Bs = T(0);
 #pragma unroll
         for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], Mth<T>::cell(kf[u]), Bs);
@@ -736,7 +734,7 @@ __device__ __forceinline__ T padded_depth_tail(const float *__restrict__ K, Padd
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
         acc = s2;
-        if ((sign & 0x80000000u) || code <= thr) break;
+        if (left || code <= thr) break;
     }
     return acc - comp;
 }
@@ -771,7 +769,7 @@ __device__ __forceinline__ T padded_depth_marks(const float *__restrict__ K, Pad
     for (;;) {
         T L[WALK_UNROLL];
         float kf[WALK_UNROLL];
-        const unsigned sign = padded_batch(K, R, L, kf);
+        const bool left = padded_batch(K, R, L, kf);
         T Bs = T(0);
 #pragma unroll
         for (int u = 0; u < WALK_UNROLL; ++u) Bs = Mth<T>::fma_(L[u], Mth<T>::cell(kf[u]), Bs);
@@ -779,7 +777,7 @@ __device__ __forceinline__ T padded_depth_marks(const float *__restrict__ K, Pad
         const T s2 = acc + y;
         comp = (s2 - acc) - y;
         acc = s2;
-        if ((sign & 0x80000000u) || (CUT && nb + 1 == n_max)) break;
+        if (left || (CUT && nb + 1 == n_max)) break;
         if (++nb % MARK_GAP == 0 && acc >= thr) {  // the same batches in every lane of a warp
             if (has_b) ia ^= 1;  // A = B
             const T b = acc - comp;
@@ -805,7 +803,7 @@ __device__ __forceinline__ bool padded_march(const float *__restrict__ K, Padded
     for (;;) {
         T L[WALK_UNROLL];
         float kf[WALK_UNROLL];
-        const unsigned sign = padded_batch(K, R, L, kf);
+        const bool left = padded_batch(K, R, L, kf);
         T dtau[WALK_UNROLL];  // each cell's optical depth, and their sum in order
         T Bs = T(0);
 #pragma unroll
@@ -839,7 +837,7 @@ __device__ __forceinline__ bool padded_march(const float *__restrict__ K, Padded
                 if (dtau[u] > T(0)) t_last = t;
             }
         }
-        if (sign & 0x80000000u) break;
+        if (left) break;
     }
     t_out = t_last;
     tau_raw = target_raw - (acc - comp);
