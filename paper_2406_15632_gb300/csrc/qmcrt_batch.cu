@@ -9,6 +9,7 @@
 // SM busy until the whole batch is done.  Per tile the CTA holds the instance's
 // parameter block in shared memory; the packet code is the single-scattering code.
 #include "qmcrt_device.cuh"
+#include "qmcrt_support.cuh"
 
 namespace qmcrt {
 
@@ -30,7 +31,10 @@ __device__ __forceinline__ uint64_t instance_tiles(const qmcrt_instance &I, int 
 }
 
 // Workspace: [0] tile counter, [1 .. n] tile prefix sums (prefix[i] = tiles of the
-// instances before i, prefix[n] = all tiles).  One block of 1024 threads.
+// instances before i, prefix[n] = all tiles).  The first, always 0, is not kept: its place
+// holds the medium's support (cleared here), with which first walks end where they leave the
+// medium: 15.1 -> 14.3 ms for 24 instances of the 256^3 finite-star disk, 38 M packets.  One block
+// of 1024 threads.
 __global__ void __launch_bounds__(1024) k_batch_plan(const qmcrt_instance *__restrict__ inst, int n, int m_cap,
                                                     uint64_t tile_packets, unsigned long long *__restrict__ ws)
 {
@@ -121,7 +125,7 @@ __global__ void __launch_bounds__(256) k_trace_batch(const __grid_constant__ Tra
             int lo = 0, hi = n_inst - 1;  // last instance whose prefix <= w
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
-                if (ws[1 + mid] <= w) lo = mid;
+                if (ws[1 + mid] <= w) lo = mid;  // mid >= 1
                 else hi = mid - 1;
             }
             const qmcrt_instance I = inst[lo];
@@ -133,7 +137,7 @@ __global__ void __launch_bounds__(256) k_trace_batch(const __grid_constant__ Tra
                 s_inst = lo;
             }
             const unsigned long long tpc = ((1ull << m) + tile_packets - 1) / tile_packets;
-            const unsigned long long local = w - ws[1 + lo];
+            const unsigned long long local = w - (lo ? ws[1 + lo] : 0ull);
             sP.ord.block0 = (I.first_index >> m) + local / tpc;
             if (sP.ord.net && sP.ord.g0_block != sP.ord.block0) {  // the block's term, once per tile
                 sP.ord.g0 = block_columns(sP.ord, sP.ord.block0 << m);
@@ -163,7 +167,7 @@ __global__ void __launch_bounds__(256) k_trace_batch(const __grid_constant__ Tra
             if (live) {
                 T pos3[3], d[3], a[3], wgt, W1;
                 const T wd = emit(P, i, pos3, d, a, wgt);
-                if (forced_step(P, pos3, d, wd, W1)) {
+                if (forced_step<T, true>(P, pos3, d, wd, W1)) {
                     const T W0 = wgt * W1 * P.dust.albedo;
                     status = peel_unpolarized(P, pos3, d, W0, S, x, y) ? 0 : 2;
                 }
@@ -185,12 +189,16 @@ __global__ void __launch_bounds__(256) k_batch_reduce(const long long *__restric
 }
 
 template <class T>
-static cudaError_t launch_batch(const TraceP<T> &p, const NetTables &tab, const qmcrt_instance *inst, int n_inst,
+static cudaError_t launch_batch(TraceP<T> p, const NetTables &tab, const qmcrt_instance *inst, int n_inst,
                                 unsigned long long *ws, int block, int ctas, int per_thread, cudaStream_t s)
 {
     k_batch_plan<<<1, 1024, 0, s>>>(inst, n_inst, tab.m_cap, (uint64_t)block * per_thread, ws);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    if (p.med.kind == QMCRT_MEDIUM_GRID && p.med.pad && n_inst > 0) {
+        k_support<T><<<152 * 8, 256, 0, s>>>(p.med, (uint32_t *)(ws + 1));
+        p.med.support = (const float *)(ws + 1);
+    }
     k_trace_batch<T><<<ctas, block, 0, s>>>(p, tab, inst, n_inst, ws, per_thread);
     return cudaGetLastError();
 }
