@@ -1,5 +1,5 @@
-// qmcrt_flow.cuh -- pieces of the learned warp shared by the layer-by-layer kernels
-// (training) and the fused forward kernel: parameter layout, one-blob features,
+// qmcrt_flow.cuh -- pieces of the learned warp shared by the fused training kernel and the
+// fused forward kernel: parameter layout, one-blob features,
 // softmax with the uniform mixture, and the piecewise-linear inverse CDF.  Both paths
 // call these same functions, so they sample identically.
 #pragma once

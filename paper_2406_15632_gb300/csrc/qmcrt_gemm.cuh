@@ -1,6 +1,6 @@
 // qmcrt_gemm.cuh -- BF16 tensor-core GEMM on the 5th-generation tensor cores (tcgen05)
-// with fused epilogues: the building block of the learned proposal's MLP (inference
-// and training).
+// with fused epilogues (qmcrt_gemm_bf16).  Its descriptor helpers and bounded mbarrier wait also
+// serve the learned proposal's fused kernels.
 //
 //   D[M x N] = A[M x K] . B[N x K]^T  (+ bias, ReLU, ReLU-mask, ...)
 //
@@ -17,13 +17,12 @@
 // skips to the end, freeing its tensor memory.  The epilogue reads the accumulator with
 // tcgen05.ld (each warp its 32 lanes = rows).
 //
-// For K <= 128 without a K split (every GEMM of the training step over the rows) a
-// persistent warp-specialised form runs instead, one CTA of 320 threads per SM: B stays in
+// For K <= 128 without a K split a persistent warp-specialised form runs instead, one CTA of 320 threads per SM: B stays in
 // shared memory, A is fetched a 128-row tile at a time by 2-D tensor copies
 // (cp.async.bulk.tensor, boxes of 8 K-elements x 128 rows, no swizzle, rows beyond M read
 // as zeros) three tiles ahead, two TMEM accumulators alternate, and the epilogue warps
-// store through a shared-memory staging tile with coalesced 16-byte stores.  The weight
-// gradients (one 128-row tile, K split over CTAs) take a tensor-copy split-K form.
+// store through a shared-memory staging tile with coalesced 16-byte stores.  One 128-row tile
+// with K split over CTAs takes a tensor-copy split-K form.
 #pragma once
 
 #include <cstdint>

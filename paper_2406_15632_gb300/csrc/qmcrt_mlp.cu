@@ -1,8 +1,7 @@
-// qmcrt_mlp.cu -- launchers of the tensor-core GEMM (qmcrt_gemm.cuh) used by the
-// learned proposal: the persistent warp-specialised tensor-copy form for K <= 128 without
-// a K split, the tensor-copy split-K form for the weight gradients (one 128-row tile,
-// FP32 vector reductions), the streaming form otherwise (and wherever a tensor map cannot
-// be made).
+// qmcrt_mlp.cu -- launchers of the tensor-core GEMM (qmcrt_gemm.cuh): the persistent
+// warp-specialised tensor-copy form for K <= 128 without a K split, the tensor-copy split-K
+// form for one 128-row tile accumulated into FP32 (vector reductions), the streaming form
+// otherwise (and wherever a tensor map cannot be made).
 #include <cudaTypedefs.h>
 
 #include "qmcrt.h"

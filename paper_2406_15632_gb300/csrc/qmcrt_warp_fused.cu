@@ -15,7 +15,7 @@
 // the tensor core works on another group's layer (three groups, 200 KB of shared memory
 // and 384 of the 512 TMEM columns: 1.29x the throughput of two).
 //
-// The arithmetic is the layer-by-layer path's (same bf16 roundings, same FP32 bias and
+// The arithmetic is the training kernel's (same bf16 roundings, same FP32 bias and
 // ReLU, same sampling functions); the feature columns that are identically zero are
 // skipped in the first layer, which adds nothing to the accumulators.
 #include <algorithm>
