@@ -41,9 +41,13 @@ struct MediumP {
     const double *sky; // optional bound map (qmcrt_sky_bound), sky_m texels per edge, for rays that start
     int sky_m;         // within sky_r2 = R^2 of the origin
     T sky_r2;
-    const float *support;      // optional: squared radii of the medium about the box centre (walk_support), in
-                               // half edges: of the ball that holds every nonzero cell, and of the cylinder along z
-    float mid[3], inv_half[3]; // the box centre, 1 / half edges
+    // optional: squared radii of the medium about the box centre (k_support), in half edges: of the
+    // ball that holds every nonzero cell, and of the cylinder along z; what support_batches needs
+    // besides: the box centre, 1 / half edges, the shortest half edge over each, half the cells of
+    // each axis, and the room left for rounding
+    const float *support;
+    T mid[3], inv_half[3];
+    float ratio[3], half_n[3], slack;
 };
 
 template <class T>
