@@ -116,8 +116,12 @@ struct SkyGeom {
 // axis state by the axis keeps it in local memory.  In float with the axes unrolled 381 us, in
 // patches of 8 x 4 texels a warp 297, with face parameters by one fused multiply-add and no cell
 // counters 200: issue-bound (76 % of the slots).  The geometry runs four cells ahead of the sum, so
-// four loads are in flight.
+// four loads are in flight.  I: a cell's index, 64 bits for grown grids beyond 2^32 cells (a fine grid
+// around a large star grows by D layers a side, whatever the grid itself may hold).  The float counts
+// of faces are exact up to 2^24 cells an axis; with more no texel passes the test of its cone below
+// (a cell is then 1.2e-7 of the longest path, the angle's own margin 1e-6).
 constexpr int SKY_BATCH = 4;
+template <class I>
 __global__ void __launch_bounds__(256) k_sky_walk(const float *__restrict__ K, const __grid_constant__ SkyGeom g,
                                                   double *__restrict__ map)
 {
@@ -174,7 +178,7 @@ __global__ void __launch_bounds__(256) k_sky_walk(const float *__restrict__ K, c
             // per axis: the first face's parameter and the spacing of the faces, faces crossed so
             // far, the next face's parameter, the index step
             float n0[3], dt[3], cnt[3] = {0.0f, 0.0f, 0.0f}, next[3], tend = inf;
-            unsigned st[3], off = 0, stride = 1;  // the tracer's grids hold at most 2^31 cells: indices modulo 2^32
+            I st[3], off = 0, stride = 1;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 // a start on a face may pick the cell on either side: the neighbourhood maximum of
@@ -190,14 +194,14 @@ __global__ void __launch_bounds__(256) k_sky_walk(const float *__restrict__ K, c
                     // no step is taken from tend on, so none leaves the box
                     tend = fminf(tend, fmaf((float)left, dt[a], n0[a]));
                 }
-                st[a] = d[a] > 0.0f ? stride : 0u - stride;
-                off += (unsigned)c * stride;
-                stride *= (unsigned)g.n[a];
+                st[a] = d[a] > 0.0f ? stride : I(0) - stride;
+                off += (I)c * stride;
+                stride *= (I)g.n[a];
             }
             float tc = t0;
             while (tc < tend) {
                 float len[SKY_BATCH];
-                unsigned at[SKY_BATCH];
+                I at[SKY_BATCH];
 #pragma unroll
                 for (int b = 0; b < SKY_BATCH; ++b) {
                     const float tn = fminf(next[0], fminf(next[1], next[2])), te = fminf(tn, tend);
@@ -293,7 +297,8 @@ cudaError_t launch_sky_bound(const float *k, int nx, int ny, int nz, const doubl
     g.room = (float)((D * hmin - 2e-6 * (1.0 + tmax)) * (1.0 - 1e-6));
     const long long patches = 6LL * ((m + 7) / 8) * ((m + 3) / 4);
     const unsigned tgrid = (unsigned)std::min<long long>((patches + 7) / 8, 152LL * 32);
-    k_sky_walk<<<tgrid, 256, 0, s>>>(A, g, map);
+    if (cells <= 1ull << 32) k_sky_walk<unsigned><<<tgrid, 256, 0, s>>>(A, g, map);
+    else k_sky_walk<unsigned long long><<<tgrid, 256, 0, s>>>(A, g, map);
     return cudaGetLastError();
 }
 
