@@ -1326,12 +1326,12 @@ __device__ __forceinline__ unsigned long long lanes_sum(unsigned mask, long long
 // add directly: summing up to 2, 4, 8 and 32 groups took 216, 225, 242 and 390 us for 10^6
 // tent-splat packets, against 215 for one, 212 for none (which costs the batch 2 %), and 228
 // with up to four groups by shuffles and 64-bit pixel keys.  Must be called by all 32 lanes.
-template <class T>
-__device__ __forceinline__ void deposit(const AccumP &A, bool valid, size_t base, unsigned pix, T I, T Q, T U)
+template <class T, class Pix = unsigned>
+__device__ __forceinline__ void deposit(const AccumP &A, bool valid, size_t base, Pix pix, T I, T Q, T U)
 {
     const int lane = threadIdx.x & 31;
     if (!__any_sync(FULL_MASK, valid)) return;
-    const unsigned peers = __match_any_sync(FULL_MASK, valid ? pix : 0xffffffffu);
+    const unsigned peers = __match_any_sync(FULL_MASK, valid ? pix : ~Pix(0));
     const bool leader = valid && ((peers & ((1u << lane) - 1u)) == 0u);
     unsigned leaders = __ballot_sync(FULL_MASK, leader);
     const size_t e = base + pix;

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(256) k_direct_star(const __grid_constant__ Tra
     const ObsP<T> &O = P.obs;
     bool in = false;
     T v = T(0);
-    unsigned e = 0;
+    unsigned long long e = 0;
     if (t < total) {
         const uint64_t pix = t / per_pix, sub = t - pix * per_pix;
         const int ix = ix0 + (int)(pix % (uint64_t)bw), iy = iy0 + (int)(pix / (uint64_t)bw);
@@ -50,11 +50,12 @@ __global__ void __launch_bounds__(256) k_direct_star(const __grid_constant__ Tra
                         (T(3.14159265358979323846) * R * R);
             const T dA = px * py / (T(S) * T(S));
             v = B * Mth<T>::exp_(-tau_to_edge(P.med, p, O.k)) * dA * weight;
-            e = (unsigned)(iy * O.nx + ix);
+            e = (unsigned long long)iy * O.nx + ix;
             in = true;
         }
     }
-    deposit<T>(P.acc, in, 0, e, v, T(0), T(0));
+    if (P.acc.plane <= 1ull << 32) deposit<T>(P.acc, in, 0, (unsigned)e, v, T(0), T(0));
+    else deposit<T, unsigned long long>(P.acc, in, 0, e, v, T(0), T(0));
 }
 
 template <class T>
