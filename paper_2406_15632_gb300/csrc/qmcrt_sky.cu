@@ -292,9 +292,10 @@ cudaError_t launch_sky_bound(const float *k, int nx, int ny, int nz, const doubl
     const double tmax = std::sqrt(far2);  // from within R of the origin to the farthest point of the grid
     g.tmax = (float)(tmax * (1.0 + 1e-6));
     // the walk's cell boundaries (face parameters recomputed from the cell index, never
-    // accumulated) sit within 2e-6 of the medium of the exact ones, taken off the room the
-    // neighbourhoods leave
-    g.room = (float)((D * hmin - 2e-6 * (1.0 + tmax)) * (1.0 - 1e-6));
+    // accumulated: about ten float roundings of coordinates up to tmax, 6e-7 of it) sit within
+    // 3e-6 tmax of the exact ones, taken off the room the neighbourhoods leave; in proportion to
+    // the box, so that a bound exists or not whatever the unit of length
+    g.room = (float)((D * hmin - 3e-6 * tmax) * (1.0 - 1e-6));
     const long long patches = 6LL * ((m + 7) / 8) * ((m + 3) / 4);
     const unsigned tgrid = (unsigned)std::min<long long>((patches + 7) / 8, 152LL * 32);
     if (cells <= 1ull << 32) k_sky_walk<unsigned><<<tgrid, 256, 0, s>>>(A, g, map);
