@@ -11,6 +11,7 @@
 #include <utility>
 
 #include "qmcrt.h"
+#include "qmcrt_block.h"
 #include "qmcrt_gemm.cuh"
 #include "qmcrt_internal.h"
 #include "qmcrt_tables.h"
@@ -452,20 +453,6 @@ struct WarpIO {
     float *log = nullptr;
 };
 
-// Threads per block of a trace whose caller names none (warps are independent: results do not
-// depend on it).  FP32: 256, whose warps trace neighbouring packets and share L1 lines (finite
-// star, 2^22 packets: 1.52 ms against 1.66 with 128 threads, 1.83 with 32), and fewer for
-// launches that would leave SMs without a block (2^12 packets on 256^3: 52 against 56 us).
-// FP64: a warp, since a slot that waits for the slowest of eight walks costs more than the
-// cache gains (50 000 star packets on 64^3: 207 against 297 us, 200 000: 798 against 863,
-// 10^5 packets of eight orders: 3.65 against 4.01 ms, 10^6 star packets the same).
-int default_block(uint64_t threads, int precision)
-{
-    int b = precision == QMCRT_PREC_F64 ? 32 : 256;
-    while (b > 32 && threads < (uint64_t)b * 304) b /= 2;
-    return b;
-}
-
 int trace_common(const qmcrt_medium *md, const qmcrt_source *src, const qmcrt_dust *du, const qmcrt_observer *ob,
                  const qmcrt_points_desc *pts, const qmcrt_trace_opts *op, const qmcrt_image *im, double *d_log,
                  void *stream, int multiple, WarpIO wio = WarpIO())
@@ -485,7 +472,7 @@ int trace_common(const qmcrt_medium *md, const qmcrt_source *src, const qmcrt_du
         P.warp_x = wio.x;
         P.warp_logj = wio.logj;
         P.train_log = wio.log;
-        const int block = op->block_size ? op->block_size : default_block(P.ord.threads, op->precision);
+        const int block = op->block_size ? op->block_size : qmcrt::default_block(P.ord.threads, op->precision == QMCRT_PREC_F64);
         return cuda_status(multiple ? qmcrt::launch_trace_multiple_f64(P, block, s)
                                     : qmcrt::launch_trace_single_f64(P, block, s),
                            "trace launch");
@@ -497,7 +484,7 @@ int trace_common(const qmcrt_medium *md, const qmcrt_source *src, const qmcrt_du
     P.warp_x = wio.x;
     P.warp_logj = wio.logj;
     P.train_log = wio.log;
-    const int block = op->block_size ? op->block_size : default_block(P.ord.threads, op->precision);
+    const int block = op->block_size ? op->block_size : qmcrt::default_block(P.ord.threads, op->precision == QMCRT_PREC_F64);
     return cuda_status(multiple ? qmcrt::launch_trace_multiple_f32(P, block, s) : qmcrt::launch_trace_single_f32(P, block, s),
                        "trace launch");
 }
@@ -550,7 +537,7 @@ int observers_common(const qmcrt_medium *md, const qmcrt_source *src, const qmcr
         if (obs[o].nx != obs[0].nx || obs[o].ny != obs[0].ny || obs[o].splat != obs[0].splat)
             return fail(QMCRT_ERR_INVALID_ARG, "observer %d: nx, ny and splat must equal observer 0's", o);
     }
-    const int block = op->block_size ? op->block_size : default_block(P.ord.threads, op->precision);
+    const int block = op->block_size ? op->block_size : qmcrt::default_block(P.ord.threads, op->precision == QMCRT_PREC_F64);
     return cuda_status(launch_observers(P, S, block, s), "trace_observers launch");
 }
 
