@@ -1320,34 +1320,44 @@ __device__ __forceinline__ unsigned long long lanes_sum(unsigned mask, long long
 }
 
 // Add (I, Q, U) at pixel pix of the image that starts `base` values into the accumulator (I
-// plane; Q, U one and two planes further); base is the same for all lanes.  Where all lanes of
-// a warp hit one pixel they are summed first (exactly, in fixed point), so that a coherent warp
-// issues one atomic per Stokes component; in FP64 up to four pixels a warp are.  Otherwise lanes
-// add directly: summing up to 2, 4, 8 and 32 groups took 216, 225, 242 and 390 us for 10^6
-// tent-splat packets, against 215 for one, 212 for none (which costs the batch 2 %), and 228
-// with up to four groups by shuffles and 64-bit pixel keys.  Must be called by all 32 lanes.
+// plane; Q, U one and two planes further); base is the same for all lanes.  Lanes of a warp that
+// hit one pixel are summed first (exactly, in fixed point), so that a coherent warp issues one
+// atomic a pixel and Stokes component: where the warp hits up to four pixels, and in fixed point
+// with three lanes or more a pixel on average.  Beyond that lanes add directly.  Atomics on few
+// pixels queue up: 2^22 tent-splat packets of the 64^3 clumpy envelope on 128^2 pixels take 0.57 ms
+// with up to four pixels summed, 0.62 with two, 1.15 with one; of 10^6 on 200^2 pixels of the 100^3 disk,
+// whose warps are a third empty, 161 us with either.  With sums from one lane a pixel on, packets of
+// the second order (few lanes left) take 7 % longer.  Must be called by all 32 lanes.
 template <class T, class Pix = unsigned>
 __device__ __forceinline__ void deposit(const AccumP &A, bool valid, size_t base, Pix pix, T I, T Q, T U)
 {
     const int lane = threadIdx.x & 31;
-    if (!__any_sync(FULL_MASK, valid)) return;
+    const unsigned vmask = __ballot_sync(FULL_MASK, valid);
+    if (vmask == 0) return;
     const unsigned peers = __match_any_sync(FULL_MASK, valid ? pix : ~Pix(0));
     const bool leader = valid && ((peers & ((1u << lane) - 1u)) == 0u);
     unsigned leaders = __ballot_sync(FULL_MASK, leader);
     const size_t e = base + pix;
     if (A.mode == QMCRT_ACCUM_I64) {
-        if (!valid) return;
         unsigned long long *dst = (unsigned long long *)A.ptr + e;
-        const long long qi = Mth<T>::to_fixed(I, A.scale), qq = Mth<T>::to_fixed(Q, A.scale),
-                        qu = Mth<T>::to_fixed(U, A.scale);
-        if ((leaders & (leaders - 1u)) == 0u) {
-            const unsigned long long a = lanes_sum(peers, qi), b = lanes_sum(peers, qq), c = lanes_sum(peers, qu);
-            if (leader) {
-                atomicAdd(dst, a);
-                atomicAdd(dst + A.plane, b);
-                atomicAdd(dst + 2 * A.plane, c);
+        const long long qi = valid ? Mth<T>::to_fixed(I, A.scale) : 0, qq = valid ? Mth<T>::to_fixed(Q, A.scale) : 0,
+                        qu = valid ? Mth<T>::to_fixed(U, A.scale) : 0;
+        const int groups = __popc(leaders);
+        if (groups <= 4 && __popc(vmask) >= 3 * groups) {
+            while (leaders) {
+                const int l = __ffs(leaders) - 1;
+                const unsigned grp = __shfl_sync(FULL_MASK, peers, l);
+                if ((grp >> lane) & 1u) {
+                    const unsigned long long a = lanes_sum(grp, qi), b = lanes_sum(grp, qq), c = lanes_sum(grp, qu);
+                    if (lane == l) {
+                        atomicAdd(dst, a);
+                        atomicAdd(dst + A.plane, b);
+                        atomicAdd(dst + 2 * A.plane, c);
+                    }
+                }
+                leaders &= leaders - 1u;
             }
-        } else {
+        } else if (valid) {
             atomicAdd(dst, (unsigned long long)qi);
             atomicAdd(dst + A.plane, (unsigned long long)qq);
             atomicAdd(dst + 2 * A.plane, (unsigned long long)qu);
