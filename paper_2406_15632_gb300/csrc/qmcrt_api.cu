@@ -324,17 +324,22 @@ int fill_trace(const qmcrt_medium *md, const qmcrt_source *src, const qmcrt_dust
             P.med.inv_h[a] = (T)(n[a] / (md->hi[a] - md->lo[a]));
             P.med.mid[a] = (T)(0.5 * (md->lo[a] + md->hi[a]));
             P.med.inv_half[a] = (T)(2.0 / (md->hi[a] - md->lo[a]));
-            P.med.half_n[a] = 0.5f * n[a];
             edge = std::min(edge, md->hi[a] - md->lo[a]);
             far = std::max(far, std::max(std::fabs(md->lo[a]), std::fabs(md->hi[a])) / (md->hi[a] - md->lo[a]));
         }
-        for (int a = 0; a < 3; ++a) P.med.ratio[a] = (float)(edge / (md->hi[a] - md->lo[a]));
+        bool flat = false;
+        for (int a = 0; a < 3; ++a) {
+            P.med.ratio[a] = (float)(edge / (md->hi[a] - md->lo[a]));
+            P.med.cells[a] = 0.5f * n[a] * P.med.ratio[a];
+            flat |= !(P.med.ratio[a] >= 1e-6f);
+        }
         // Room in the squared radii of the support: 2e-5 for the float arithmetic of support_batches
         // (a few 1e-6), and what a point near a face may be off by, in half edges: faces and
         // centre are rounded to T where the box lies, four roundings of |lo| or |hi| at most.  Where
-        // that is a quarter of the half edge nothing is cut.
+        // that is a quarter of the half edge nothing is cut, nor in a box of edges 1e6 apart (the
+        // squares of the ratios have to stay in a float's range).
         const double off = 4.0 * std::numeric_limits<T>::epsilon() * far;
-        P.med.slack = off < 0.25 ? (float)(2e-5 + 8.0 * off + 4.0 * off * off) : std::numeric_limits<float>::infinity();
+        P.med.slack = off < 0.25 && !flat ? (float)(2e-5 + 8.0 * off + 4.0 * off * off) : std::numeric_limits<float>::infinity();
         if (md->pad != 0 && md->pad < QMCRT_MIN_PAD)
             return fail(QMCRT_ERR_INVALID_ARG, "pad %d: 0 or at least %d", md->pad, QMCRT_MIN_PAD);
         const int px = md->nx + 2 * md->pad, py = md->ny + 2 * md->pad, pz = md->nz + 2 * md->pad;

@@ -666,9 +666,9 @@ template <class T>
 __device__ __forceinline__ unsigned support_batches(const MediumP<T> &G, const T p[3], const T d[3],
                                                     const PaddedRay<T> &R)
 {
-    // Everything in half edges of the box, the ray's parameter in the time its fastest axis takes for
-    // one: no unit of length enters (e = d / half edge would: its square leaves the range of a
-    // float for edges beyond 1e19 or below 1e-19).
+    // Positions in half edges of the box, the ray's parameter in the shortest of them: no unit of
+    // length enters (the square of d / half edge would leave the range of a float for edges beyond
+    // 1e19 or below 1e-19).
     const float ball = __ldg(G.support) + G.slack, cyl = __ldg(G.support + 1) + G.slack;
     float q[3], e[3];
 #pragma unroll
@@ -676,15 +676,10 @@ __device__ __forceinline__ unsigned support_batches(const MediumP<T> &G, const T
         q[a] = (float)((p[a] - G.mid[a]) * G.inv_half[a]);
         e[a] = (float)d[a] * G.ratio[a];
     }
-    const float fast = fmaxf(fabsf(e[0]), fmaxf(fabsf(e[1]), fabsf(e[2])));
-    if (!(fast > 1e-30f)) return 0xffffffffu;
-    const float inv = 1.0f / fast;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) e[a] *= inv;
     // far root of |q + t e|^2 = r^2; a ray that misses, or leaves behind its start, has none ahead
     auto leaves = [](float A, float B, float C) {
         const float disc = B * B - A * C;
-        if (A < 1e-20f) return C > 0.0f ? 0.0f : __int_as_float(0x7f800000);  // moves 1e-10 at most: inside or out
+        if (A < 1e-30f) return C > 0.0f ? 0.0f : __int_as_float(0x7f800000);  // moves 1e-8 at most: inside or out
         return disc > 0.0f ? fmaxf((sqrtf(disc) - B) / A, 0.0f) : 0.0f;
     };
     const float A2 = e[0] * e[0] + e[1] * e[1], B2 = q[0] * e[0] + q[1] * e[1], C2 = q[0] * q[0] + q[1] * q[1];
@@ -697,7 +692,7 @@ __device__ __forceinline__ unsigned support_batches(const MediumP<T> &G, const T
     float cells = 2.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a)
-        cells += fmaxf(t * (fabsf(e[a]) * G.half_n[a]) - (float)(s[a] * G.inv_h[a]) * fabsf((float)d[a]) + 1.0f, 0.0f);
+        cells += fmaxf((t * G.cells[a] - (float)(s[a] * G.inv_h[a])) * fabsf((float)d[a]) + 1.0f, 0.0f);
     return __float2uint_ru(cells * (1.0f / WALK_UNROLL));
 }
 

@@ -43,11 +43,11 @@ struct MediumP {
     T sky_r2;
     // optional: squared radii of the medium about the box centre (k_support), in half edges: of the
     // ball that holds every nonzero cell, and of the cylinder along z; what support_batches needs
-    // besides: the box centre, 1 / half edges, the shortest half edge over each, half the cells of
-    // each axis, and the room left for rounding
+    // besides: the box centre, 1 / half edges, the shortest half edge over each, the cells of each
+    // axis on that length, and the room left for rounding
     const float *support;
     T mid[3], inv_half[3];
-    float ratio[3], half_n[3], slack;
+    float ratio[3], cells[3], slack;
 };
 
 template <class T>
