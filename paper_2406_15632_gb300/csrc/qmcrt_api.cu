@@ -314,7 +314,7 @@ int fill_trace(const qmcrt_medium *md, const qmcrt_source *src, const qmcrt_dust
         if ((double)md->nx * md->ny * md->nz > 2147483647.0)
             return fail(QMCRT_ERR_INVALID_ARG, "grid larger than 2^31 cells");
         const int n[3] = {md->nx, md->ny, md->nz};
-        double edge = std::numeric_limits<double>::infinity(), far = 0.0;  // shortest edge; farthest face, in edges
+        double edge = std::numeric_limits<double>::infinity(), longest = 0.0, far = 0.0;  // far: the farthest face, in edges
         for (int a = 0; a < 3; ++a) {
             if (!(md->hi[a] > md->lo[a])) return fail(QMCRT_ERR_INVALID_ARG, "grid box axis %d is empty", a);
             P.med.n[a] = n[a];
@@ -322,24 +322,17 @@ int fill_trace(const qmcrt_medium *md, const qmcrt_source *src, const qmcrt_dust
             P.med.hi[a] = (T)md->hi[a];
             P.med.h[a] = (T)((md->hi[a] - md->lo[a]) / n[a]);
             P.med.inv_h[a] = (T)(n[a] / (md->hi[a] - md->lo[a]));
-            P.med.mid[a] = (T)(0.5 * (md->lo[a] + md->hi[a]));
-            P.med.inv_half[a] = (T)(2.0 / (md->hi[a] - md->lo[a]));
+            P.med.mid[a] = (float)(0.5 * (md->lo[a] + md->hi[a]));
+            longest = std::max(longest, md->hi[a] - md->lo[a]);
             edge = std::min(edge, md->hi[a] - md->lo[a]);
             far = std::max(far, std::max(std::fabs(md->lo[a]), std::fabs(md->hi[a])) / (md->hi[a] - md->lo[a]));
         }
-        bool flat = false;
-        for (int a = 0; a < 3; ++a) {
-            P.med.ratio[a] = (float)(edge / (md->hi[a] - md->lo[a]));
-            P.med.cells[a] = 0.5f * n[a] * P.med.ratio[a];
-            flat |= !(P.med.ratio[a] >= 1e-6f);
-        }
-        // Room in the squared radii of the support: 2e-5 for the float arithmetic of support_batches
-        // (a few 1e-6), and what a point near a face may be off by, in half edges: faces and
-        // centre are rounded to T where the box lies, four roundings of |lo| or |hi| at most.  Where
-        // that is a quarter of the half edge nothing is cut, nor in a box of edges 1e6 apart (the
-        // squares of the ratios have to stay in a float's range).
-        const double off = 4.0 * std::numeric_limits<T>::epsilon() * far;
-        P.med.slack = off < 0.25 && !flat ? (float)(2e-5 + 8.0 * off + 4.0 * off * off) : std::numeric_limits<float>::infinity();
+        // scale^2 is about the shortest half edge (support_batches).  No cut (inv_half = 0) beyond 1e24
+        // or below 1e-24 units, in a box of edges a factor of 1000 apart, or far from the origin, where
+        // the float rounding of a position (a few roundings of |lo| or |hi|) would outgrow its room.
+        const double scale = std::exp2(std::floor(0.5 * std::log2(0.5 * edge)));
+        const bool cut = edge > 1e-24 && edge < 1e24 && longest < 1000.0 * edge && far < 2.5;
+        for (int a = 0; a < 3; ++a) P.med.inv_half[a] = cut ? (float)(2.0 * scale / (md->hi[a] - md->lo[a])) : 0.0f;
         if (md->pad != 0 && md->pad < QMCRT_MIN_PAD)
             return fail(QMCRT_ERR_INVALID_ARG, "pad %d: 0 or at least %d", md->pad, QMCRT_MIN_PAD);
         const int px = md->nx + 2 * md->pad, py = md->ny + 2 * md->pad, pz = md->nz + 2 * md->pad;

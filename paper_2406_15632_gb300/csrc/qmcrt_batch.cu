@@ -195,8 +195,8 @@ static cudaError_t launch_batch(TraceP<T> p, const NetTables &tab, const qmcrt_i
     k_batch_plan<<<1, 1024, 0, s>>>(inst, n_inst, tab.m_cap, (uint64_t)block * per_thread, ws);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (p.med.kind == QMCRT_MEDIUM_GRID && p.med.pad && n_inst > 0) {
-        k_support<T><<<152 * 8, 256, 0, s>>>(p.med, (uint32_t *)(ws + 1));
+    if (p.med.kind == QMCRT_MEDIUM_GRID && p.med.pad && p.med.inv_half[0] > 0.0f) {
+        k_support<T><<<152 * 8, 256, 0, s>>>(p.med, support_scale2(p.med), (uint32_t *)(ws + 1));
         p.med.support = (const float *)(ws + 1);
     }
     k_trace_batch<T><<<ctas, block, 0, s>>>(p, tab, inst, n_inst, ws, per_thread);

@@ -666,33 +666,31 @@ template <class T>
 __device__ __forceinline__ unsigned support_batches(const MediumP<T> &G, const T p[3], const T d[3],
                                                     const PaddedRay<T> &R)
 {
-    // Positions in half edges of the box, the ray's parameter in the shortest of them: no unit of
-    // length enters (the square of d / half edge would leave the range of a float for edges beyond
-    // 1e19 or below 1e-19).
-    const float ball = __ldg(G.support) + G.slack, cyl = __ldg(G.support + 1) + G.slack;
+    // Positions and directions are in half edges times scale (inv_half and the radii hold it), a
+    // length's square root: A is about 1 / length, C a length and the discriminant free of units, so
+    // that none takes them out of a float's range.  The radii hold the room for rounding.
+    const float ball = __ldg(G.support), cyl = __ldg(G.support + 1);
     float q[3], e[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        q[a] = (float)((p[a] - G.mid[a]) * G.inv_half[a]);
-        e[a] = (float)d[a] * G.ratio[a];
+        q[a] = ((float)p[a] - G.mid[a]) * G.inv_half[a];
+        e[a] = (float)d[a] * G.inv_half[a];
     }
     // far root of |q + t e|^2 = r^2; a ray that misses, or leaves behind its start, has none ahead
     auto leaves = [](float A, float B, float C) {
         const float disc = B * B - A * C;
-        if (A < 1e-30f) return C > 0.0f ? 0.0f : __int_as_float(0x7f800000);  // moves 1e-8 at most: inside or out
+        if (A == 0.0f) return C > 0.0f ? 0.0f : __int_as_float(0x7f800000);
         return disc > 0.0f ? fmaxf((sqrtf(disc) - B) / A, 0.0f) : 0.0f;
     };
     const float A2 = e[0] * e[0] + e[1] * e[1], B2 = q[0] * e[0] + q[1] * e[1], C2 = q[0] * q[0] + q[1] * q[1];
     float t = leaves(A2 + e[2] * e[2], B2 + q[2] * e[2], C2 + q[2] * q[2] - ball);
-    if (cyl < 2.0f) t = fminf(t, leaves(A2, B2, C2 - cyl));
+    if (cyl < 1e37f) t = fminf(t, leaves(A2, B2, C2 - cyl));
     if (t == 0.0f) return 0u;
-    // faces crossed per axis until t, one more each for the crossing at hand, and one for rounding;
-    // s |d| / h is the part of a cell left before the first face (NaN on an axis never crossed: 0)
-    const T s[3] = {R.X.s, R.Y.s, R.Z.s};
+    // faces crossed per axis until t, one more each for the crossing at hand, and one for rounding
     float cells = 2.0f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-        cells += fmaxf((t * G.cells[a] - (float)(s[a] * G.inv_h[a])) * fabsf((float)d[a]) + 1.0f, 0.0f);
+    cells += fmaxf((t - (float)R.X.s) * fabsf((float)d[0] * (float)G.inv_h[0]) + 1.0f, 0.0f);
+    cells += fmaxf((t - (float)R.Y.s) * fabsf((float)d[1] * (float)G.inv_h[1]) + 1.0f, 0.0f);
+    cells += fmaxf((t - (float)R.Z.s) * fabsf((float)d[2] * (float)G.inv_h[2]) + 1.0f, 0.0f);
     return __float2uint_ru(cells * (1.0f / WALK_UNROLL));
 }
 

@@ -6,11 +6,20 @@
 
 namespace qmcrt {
 
+// scale^2 of a medium's support (see support_batches), to a few float roundings.
+template <class T>
+static float support_scale2(const MediumP<T> &G)
+{
+    const double s = 0.5 * G.n[0] * (double)G.h[0] * (double)G.inv_half[0];
+    return (float)(s * s);
+}
+
 // Support of a padded grid: the largest squared distance, in half edges of the box, of a nonzero
 // cell's farthest corner from the box centre (ball) and from the line along z through it
-// (cylinder).  `support`: two words, cleared by the caller.  One read of the grid a run.
+// (cylinder), times scale2.  `support`: two words, cleared by the caller.  One read of the grid a run.
 template <class T>
-static __global__ void __launch_bounds__(256) k_support(const __grid_constant__ MediumP<T> G, uint32_t *support)
+static __global__ void __launch_bounds__(256) k_support(const __grid_constant__ MediumP<T> G, float scale2,
+                                                       uint32_t *support)
 {
     const int lane = threadIdx.x & 31, rows = G.n[1] * G.n[2], warps = gridDim.x * 8;
     const float per[3] = {2.0f / G.n[0], 2.0f / G.n[1], 2.0f / G.n[2]};  // cell edges in half edges of the box
@@ -45,8 +54,13 @@ static __global__ void __launch_bounds__(256) k_support(const __grid_constant__ 
         atomicMax(&s_max[1], c);
     }
     __syncthreads();
-    if (threadIdx.x < 2 && s_max[threadIdx.x] > *(volatile uint32_t *)(support + threadIdx.x))
-        atomicMax(support + threadIdx.x, s_max[threadIdx.x]);
+    if (threadIdx.x < 2 && s_max[threadIdx.x]) {
+        // no cut where it takes in the whole box (a corner, a column at an edge); 2e-5 for the
+        // float rounding of the radii, of positions and of directions
+        const float r2 = __uint_as_float(s_max[threadIdx.x]) + 2e-5f;
+        const uint32_t bits = __float_as_uint(r2 < (threadIdx.x ? 2.0f : 3.0f) ? r2 * scale2 : 3e38f);
+        if (bits > *(volatile uint32_t *)(support + threadIdx.x)) atomicMax(support + threadIdx.x, bits);
+    }
 }
 
 }  // namespace qmcrt

@@ -398,9 +398,9 @@ cudaError_t launch_wave(TraceP<T> P, void *ws, uint64_t cap, int sms, cudaStream
     cudaError_t e = cudaMemsetAsync(W.count, 0, WV_TAIL_BYTES, s);
     if (e == cudaSuccess && P.max_orders > 1) e = cudaMemsetAsync(W.hist, 0, (size_t)buckets * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    if (P.med.kind == QMCRT_MEDIUM_GRID && P.med.pad) {
+    if (P.med.kind == QMCRT_MEDIUM_GRID && P.med.pad && P.med.inv_half[0] > 0.0f) {
         uint32_t *support = (uint32_t *)(W.count + 66);
-        k_support<T><<<(unsigned)std::max(1, sms * 8), 256, 0, s>>>(P.med, support);
+        k_support<T><<<(unsigned)std::max(1, sms * 8), 256, 0, s>>>(P.med, support_scale2(P.med), support);
         P.med.support = (const float *)support;
     }
     const uint64_t threads = (P.ord.threads + 31) & ~31ull;

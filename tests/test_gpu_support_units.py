@@ -14,7 +14,8 @@ Z, Y, X = np.meshgrid(c, c, c, indexing="ij")
 BALL = (X * X + Y * Y + Z * Z < 0.8) * np.random.default_rng(2).uniform(0.5, 4.0, size=(N, N, N))
 BOXES = {"1e22": ((-1e22,) * 3, (1e22,) * 3), "3e22": ((-3e22,) * 3, (3e22,) * 3), "1e-20": ((-1e-20,) * 3, (1e-20,) * 3),
          "flat": ((-1.0, -1e3, -1e-2), (1.0, 1e3, 1e-2)),
-         "flat 1e18": ((-1e18, -1e21, -1e16), (1e18, 1e21, 1e16)), "needle": ((-1.0, -1.0, -1e8), (1.0, 1.0, 1e8)), "unit": ((-1.0,) * 3, (1.0,) * 3)}
+         "flat 1e18": ((-1e18, -1e21, -1e16), (1e18, 1e21, 1e16)), "needle": ((-1.0, -1.0, -1e8), (1.0, 1.0, 1e8)),
+         "slab 3e20": ((-1e20, -3e20, -1e18), (1e20, 3e20, 1e18)), "corner": ((-0.01,) * 3, (1.99,) * 3), "unit": ((-1.0,) * 3, (1.0,) * 3)}
 
 
 @pytest.fixture(scope="module")
