@@ -33,19 +33,38 @@ __device__ __forceinline__ uint64_t instance_tiles(const qmcrt_instance &I, int 
 // Workspace: [0] tile counter, [1 .. n] tile prefix sums (prefix[i] = tiles of the
 // instances before i, prefix[n] = all tiles).  The first, always 0, is not kept: its place
 // holds the medium's support (cleared here), with which first walks end where they leave the
-// medium: 15.1 -> 14.3 ms for 24 instances of the 256^3 finite-star disk, 38 M packets.  One block
-// of 1024 threads.
+// medium: 15.1 -> 14.3 ms for 24 instances of the 256^3 finite-star disk, 38 M packets.  The cut
+// costs a read of the grid, which few packets do not pay for: it is left out (the support set
+// to everything) below cells / 2048 packets, unless an instance has 8192, whose longest walks
+// then count.  Start to end in us, without and with it: 256^3 with 2^10 packets 209 / 241, 2^12 258 / 281,
+// 2^13 340 / 319, 24 x 2^8 147 / 177, 24 x 2^10 361 / 346; 512^3 with 2^10 498 / 779, 2^13 843 / 806,
+// 24 x 2^10 644 / 809, 24 x 2^12 1010 / 948.  One block of 1024 threads.
 __global__ void __launch_bounds__(1024) k_batch_plan(const qmcrt_instance *__restrict__ inst, int n, int m_cap,
-                                                    uint64_t tile_packets, unsigned long long *__restrict__ ws)
+                                                    uint64_t tile_packets, uint64_t cells,
+                                                    unsigned long long *__restrict__ ws)
 {
     __shared__ unsigned long long part[1024];
+    __shared__ unsigned s_all, s_most;  // packets of all instances, of the largest (up to 2^20 a thread)
     const int t = threadIdx.x;
     const int per = (n + 1023) / 1024;
     const int a = min(n, t * per), b = min(n, a + per);
     unsigned long long s = 0;
-    for (int i = a; i < b; ++i) s += instance_tiles(inst[i], m_cap, tile_packets);
+    unsigned all = 0, most = 0;
+    for (int i = a; i < b; ++i) {
+        s += instance_tiles(inst[i], m_cap, tile_packets);
+        const unsigned c = (unsigned)min((unsigned long long)inst[i].count, 1ull << 20);
+        all = min(all + c, 1u << 20);
+        most = max(most, c);
+    }
     part[t] = s;
+    if (t == 0) s_all = s_most = 0u;
     __syncthreads();
+    all = __reduce_add_sync(FULL_MASK, all);
+    most = __reduce_max_sync(FULL_MASK, most);
+    if ((t & 31) == 0 && all) {
+        atomicAdd(&s_all, all);
+        atomicMax(&s_most, most);
+    }
     for (int off = 1; off < 1024; off <<= 1) {  // inclusive scan (Hillis-Steele)
         const unsigned long long v = t >= off ? part[t - off] : 0ull;
         __syncthreads();
@@ -54,11 +73,16 @@ __global__ void __launch_bounds__(1024) k_batch_plan(const qmcrt_instance *__res
     }
     unsigned long long run = t ? part[t - 1] : 0ull;
     for (int i = a; i < b; ++i) {
-        ws[1 + i] = run;
+        if (i) ws[1 + i] = run;
         run += instance_tiles(inst[i], m_cap, tile_packets);
     }
     if (t == 1023) ws[1 + n] = part[1023];
-    if (t == 0) ws[0] = 0ull;
+    if (t == 0) {
+        ws[0] = 0ull;
+        const bool few = s_most < 8192 && s_all < cells / 2048;  // at most 2^20
+        const unsigned long long none = __float_as_uint(SUPPORT_ALL);
+        ws[1] = few ? none << 32 | none : 0ull;
+    }
 }
 
 template <class T>
@@ -192,7 +216,8 @@ template <class T>
 static cudaError_t launch_batch(TraceP<T> p, const NetTables &tab, const qmcrt_instance *inst, int n_inst,
                                 unsigned long long *ws, int block, int ctas, int per_thread, cudaStream_t s)
 {
-    k_batch_plan<<<1, 1024, 0, s>>>(inst, n_inst, tab.m_cap, (uint64_t)block * per_thread, ws);
+    const uint64_t cells = (uint64_t)p.med.n[0] * p.med.n[1] * p.med.n[2];
+    k_batch_plan<<<1, 1024, 0, s>>>(inst, n_inst, tab.m_cap, (uint64_t)block * per_thread, cells, ws);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (p.med.kind == QMCRT_MEDIUM_GRID && p.med.pad && p.med.inv_half[0] > 0.0f) {

@@ -6,6 +6,8 @@
 
 namespace qmcrt {
 
+constexpr float SUPPORT_ALL = 3e38f;  // radii beyond every box: no cut
+
 // scale^2 of a medium's support (see support_batches), to a few float roundings.
 template <class T>
 static float support_scale2(const MediumP<T> &G)
@@ -21,6 +23,9 @@ template <class T>
 static __global__ void __launch_bounds__(256) k_support(const __grid_constant__ MediumP<T> G, float scale2,
                                                        uint32_t *support)
 {
+    // already the whole box: nothing to find (set by the caller, or by a block that met a corner cell,
+    // which sets both; read through L1: 1216 blocks at one word of L2 take 2 us, and an old value will do)
+    if (*support == __float_as_uint(SUPPORT_ALL)) return;
     const int lane = threadIdx.x & 31, rows = G.n[1] * G.n[2], warps = gridDim.x * 8;
     const float per[3] = {2.0f / G.n[0], 2.0f / G.n[1], 2.0f / G.n[2]};  // cell edges in half edges of the box
     auto far2 = [&](int first, int last, int axis) {  // squared distance of the farther end of a run of cells
@@ -58,7 +63,7 @@ static __global__ void __launch_bounds__(256) k_support(const __grid_constant__ 
         // no cut where it takes in the whole box (a corner, a column at an edge); 2e-5 for the
         // float rounding of the radii, of positions and of directions
         const float r2 = __uint_as_float(s_max[threadIdx.x]) + 2e-5f;
-        const uint32_t bits = __float_as_uint(r2 < (threadIdx.x ? 2.0f : 3.0f) ? r2 * scale2 : 3e38f);
+        const uint32_t bits = __float_as_uint(r2 < (threadIdx.x ? 2.0f : 3.0f) ? r2 * scale2 : SUPPORT_ALL);
         if (bits > *(volatile uint32_t *)(support + threadIdx.x)) atomicMax(support + threadIdx.x, bits);
     }
 }

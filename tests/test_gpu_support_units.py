@@ -81,3 +81,24 @@ def test_box_beside_the_star(Q, precision):
     torch.cuda.synchronize()
     assert torch.equal(a, b)
     assert bool((a[:, 1:] != 0).any())
+
+
+@pytest.mark.parametrize("sizes", [(1,), (2047,), (2048,), (100, 8191), (8192, 0, 5), (0, 0), (700, 700, 700)])
+def test_small_batches_with_and_without_the_cut(Q, sizes):
+    """Batches on both sides of the size from which the support is looked for, one after another in one
+    workspace."""
+    import torch
+
+    p = _problem("unit", source="sphere", star_r=0.1)
+    sc = Q.Scene(p)
+    inst = [S.Instance(theta_obs=0.3 * k, albedo=0.7, g=0.4, kscale=0.5 + k, n_packets=n, first_index=9)
+            for k, n in enumerate(sizes)]
+    b = Q.Batch(p, inst, frac_bits=36, scene=sc)
+    for _ in range(2):
+        b.run()
+        got = b.accum.clone()
+        b.ws.fill_(-1)
+    b.run_each()
+    torch.cuda.synchronize()
+    assert torch.equal(got, b.accum)
+    assert bool((got != 0).any()) == (max(sizes) > 0)
