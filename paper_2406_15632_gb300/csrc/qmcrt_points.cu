@@ -18,17 +18,20 @@ namespace qmcrt {
 // high four bits) that hold for every tile.
 constexpr int PTS_BITS = 8, PTS_TILE = 1 << PTS_BITS, PTS_HALF = 1 << (PTS_BITS / 2);
 constexpr uint64_t PTS_CTAS = 152 * 8;  // blocks of 256 threads resident at once
+constexpr uint64_t PTS_FEW = 38;        // up to so many tiles, eight blocks take one: two blocks an SM
+constexpr unsigned PTS_PARTS = 8;
 
 // Sobol direction numbers in global memory: lanes of a warp read them for different
 // dimensions, which constant memory would serve one address at a time.
 static __device__ const uint32_t d_sobol_v[QMCRT_GEN_DIMS][32] = QMCRT_GEN_SOBOL_V_INIT;
 
-// XOR of the columns of dimension d over the set bits of g.
-__device__ __forceinline__ uint32_t xor_columns(const uint32_t (*V)[32], int d, uint32_t g)
+// x * 2^-32 in FP64, exact, by its bits: the FP64 pipe (1/64 of the float rate) takes one conversion and
+// one product a value otherwise, which bounds points of few dimensions.
+__device__ __forceinline__ double unit_f64(uint32_t x)
 {
-    uint32_t x = 0;
-    for (; g; g &= g - 1u) x ^= __ldg(&V[d][__ffs(g) - 1]);
-    return x;
+    const int n = __clz((int)x);
+    const uint32_t f = x << (n & 31);  // the leading bit at 31: 1.xxx times 2^(-1 - n)
+    return __hiloint2double(x ? (int)((f >> 11) + ((uint32_t)(1021 - n) << 20)) : 0, (int)(f << 21));
 }
 
 template <int FMT>
@@ -36,7 +39,7 @@ __device__ __forceinline__ void put_u32(void *out, uint64_t e, uint32_t x)
 {
     if (FMT == QMCRT_FMT_U32) ((uint32_t *)out)[e] = x;
     else if (FMT == QMCRT_FMT_F32) ((float *)out)[e] = Mth<float>::from_u32(x);
-    else ((double *)out)[e] = Mth<double>::from_u32(x);
+    else ((double *)out)[e] = unit_f64(x);
 }
 
 // Four consecutive values, at an element index that is a multiple of four.
@@ -51,18 +54,22 @@ __device__ __forceinline__ void put4_u32(void *out, uint64_t e, uint4 w)
                         Mth<float>::from_u32(w.w));
     } else {
         double2 *o = reinterpret_cast<double2 *>((double *)out + e);
-        o[0] = make_double2(Mth<double>::from_u32(w.x), Mth<double>::from_u32(w.y));
-        o[1] = make_double2(Mth<double>::from_u32(w.z), Mth<double>::from_u32(w.w));
+        o[0] = make_double2(unit_f64(w.x), unit_f64(w.y));
+        o[1] = make_double2(unit_f64(w.z), unit_f64(w.w));
     }
 }
 
 // The elements [e0, e1) of a tile's [rows][dims] block, thread by thread: f(e, j, d) for
-// element e = j dims + d; j and d advance by the block's stride without a division.
+// element e = j dims + d; j and d advance by the block's stride without a division.  The first of
+// them from a float quotient, exact here: e < 2^17 and a half is added, so the quotient is 0.5 / dims
+// off a whole number at least, and its rounding 2^-6 / dims at most.
 template <class F>
 __device__ __forceinline__ void tile_elements(uint32_t e0, uint32_t e1, uint32_t dims, F f)
 {
-    const uint32_t sj = blockDim.x / dims, sd = blockDim.x - sj * dims;
-    uint32_t e = e0 + threadIdx.x, j = e / dims, d = e - j * dims;
+    const float per = 1.0f / (float)dims;
+    auto quotient = [&](uint32_t v) { return (uint32_t)(((float)v + 0.5f) * per); };
+    const uint32_t sj = quotient(blockDim.x), sd = blockDim.x - sj * dims;
+    uint32_t e = e0 + threadIdx.x, j = quotient(e), d = e - j * dims;
     for (; e < e1; e += blockDim.x) {
         f(e, j, d);
         j += sj;
@@ -77,33 +84,57 @@ __device__ __forceinline__ void tile_elements(uint32_t e0, uint32_t e1, uint32_t
 // Sobol, Owen-scrambled Sobol and Niederreiter points.  VEC: a thread takes four consecutive
 // dimensions, with 16-byte reads of the tables and stores; for dimension counts that are a
 // multiple of four (every row, and so every table row, then starts on 16 bytes) and an output
-// on a 16-byte boundary.  2^20 x 80 Sobol coordinates in FP32 (49 us at the copy rate):
-// 35 ms -> 105 us an element at a time, 77 us four at a time (4.4 TB/s).
+// on a 16-byte boundary.  `parts` blocks share a tile of a small output (PTS_PARTS).  2^20 x 80 Sobol
+// coordinates in FP32 (49 us at the copy rate): 35 ms one element a thread, 105 us by tiles an element at
+// a time, 77 four at a time, 57 (5.9 TB/s) with the base's bits over the lanes of a warp instead of one
+// after the other in a thread, which also held up few dimensions (2^24 x 1: 78 -> 60 us) and, in the tables,
+// short outputs of many (100 x 256 in FP64: 35 us, 12 so).
 template <int KIND, int FMT, bool VEC>
 __global__ void __launch_bounds__(256) k_points_net(const __grid_constant__ PointsP P, uint64_t first, uint64_t count,
-                                                    void *out)
+                                                    void *out, uint32_t parts)
 {
     extern __shared__ uint4 s_tab4[];  // [PTS_HALF][dims] low bits, the same for the high bits, [dims] base, seeds
     uint32_t *const s_tab = reinterpret_cast<uint32_t *>(s_tab4);
     const uint32_t (*V)[32] = KIND == QMCRT_NIEDERREITER ? d_nied_v : d_sobol_v;
     const uint32_t dims = (uint32_t)P.dims;
+    const uint32_t lane = threadIdx.x & 31;
     uint32_t *lo = s_tab, *hi = lo + PTS_HALF * dims, *bs = hi + PTS_HALF * dims, *sd = bs + dims;
-    for (uint32_t q = threadIdx.x; q < PTS_HALF * dims; q += blockDim.x) {
-        const uint32_t a = q / dims, d = q - a * dims, b = a << (PTS_BITS / 2);
-        lo[q] = xor_columns(V, d, KIND == QMCRT_NIEDERREITER ? a : a ^ (a >> 1));
-        hi[q] = xor_columns(V, d, KIND == QMCRT_NIEDERREITER ? b : b ^ (b >> 1));
+    // a thread a dimension and half: the columns of four bits, their 16 sums by one XOR each
+    for (uint32_t q = threadIdx.x; q < 2 * dims; q += blockDim.x) {
+        const uint32_t half = q >= dims, d = q - half * dims;
+        uint32_t *tab = half ? hi : lo, col[PTS_BITS / 2], x[PTS_HALF];
+#pragma unroll
+        for (int k = 0; k < PTS_BITS / 2; ++k) {
+            const uint32_t bit = half * (PTS_BITS / 2) + k;
+            col[k] = __ldg(&V[d][bit]);  // through the Gray code a bit is its own column and the one below
+            if (KIND != QMCRT_NIEDERREITER && bit) col[k] ^= __ldg(&V[d][bit - 1]);
+        }
+        x[0] = 0;
+        tab[d] = 0;
+#pragma unroll
+        for (int a = 1; a < PTS_HALF; ++a) {
+            const int low = a & -a;
+            x[a] = x[a ^ low] ^ col[low == 1 ? 0 : low == 2 ? 1 : low == 4 ? 2 : 3];
+            tab[a * dims + d] = x[a];
+        }
     }
     if (KIND == QMCRT_SOBOL_OWEN)
         for (uint32_t d = threadIdx.x; d < dims; d += blockDim.x) sd[d] = owen_seed(P.seed, (int)d);
     const uint64_t t0 = first >> PTS_BITS, t1 = (first + count - 1) >> PTS_BITS;
-    for (uint64_t t = t0 + blockIdx.x; t <= t1; t += gridDim.x) {
+    const uint32_t part = blockIdx.x % parts, per_part = PTS_TILE / parts;
+    for (uint64_t t = t0 + blockIdx.x / parts; t <= t1; t += gridDim.x / parts) {
         const uint64_t base = t << PTS_BITS;
         const uint32_t b32 = (uint32_t)base, g = KIND == QMCRT_NIEDERREITER ? b32 : b32 ^ (b32 >> 1);
         __syncthreads();  // the last tile's elements are done with bs
-        for (uint32_t d = threadIdx.x; d < dims; d += blockDim.x) bs[d] = xor_columns(V, d, g);
+        // a warp a dimension, a lane a bit
+        for (uint32_t d = threadIdx.x / 32; d < dims; d += blockDim.x / 32) {
+            const uint32_t x = __reduce_xor_sync(FULL_MASK, (g >> lane) & 1u ? __ldg(&V[d][lane]) : 0u);
+            if (lane == 0) bs[d] = x;
+        }
         __syncthreads();
-        const uint32_t j0 = base < first ? (uint32_t)(first - base) : 0u;
-        const uint32_t j1 = (uint32_t)min((uint64_t)PTS_TILE, first + count - base);
+        const uint32_t j0 = max(base < first ? (uint32_t)(first - base) : 0u, part * per_part);
+        const uint32_t j1 = min((uint32_t)min((uint64_t)PTS_TILE, first + count - base), (part + 1) * per_part);
+        if (j0 >= j1) continue;  // uniform
         const uint64_t off = (base - first) * dims;  // modulo 2^64: element e of the tile is off + e
         if (VEC) {
             const uint32_t quads = dims / 4;
@@ -159,10 +190,12 @@ __global__ void __launch_bounds__(256) k_points_philox(const __grid_constant__ P
 // Halton, Hammersley and Faure points (values, no integer form), one element a thread: bound by
 // the digit expansions and the FP64 division that rounds each fraction (digits by multiplication
 // instead of division, and longer-lived blocks, were 0 to 15 % slower).
-template <int FMT>
-__global__ void __launch_bounds__(256) k_points_digits(const __grid_constant__ PointsP P, uint64_t first,
+template <int KIND, int FMT>
+__global__ void __launch_bounds__(256) k_points_digits(const __grid_constant__ PointsP base, uint64_t first,
                                                        uint64_t count, void *out)
 {
+    PointsP P = base;
+    P.kind = KIND;
     const uint64_t total = count * (uint64_t)P.dims;
     for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (uint64_t)gridDim.x * blockDim.x) {
@@ -240,12 +273,13 @@ template <int KIND, int FMT>
 static void launch_points_net(const PointsP &p, uint64_t first, uint64_t count, void *out, cudaStream_t s)
 {
     const uint64_t tiles = ((first + count - 1) >> PTS_BITS) - (first >> PTS_BITS) + 1;
-    const unsigned grid = (unsigned)(tiles < PTS_CTAS ? tiles : PTS_CTAS);
+    const unsigned parts = tiles <= PTS_FEW && p.dims >= 16 ? PTS_PARTS : 1;
+    const unsigned grid = (unsigned)(tiles < PTS_CTAS ? tiles : PTS_CTAS) * parts;
     const size_t smem = (2 * PTS_HALF + 2) * (size_t)p.dims * sizeof(uint32_t);  // 34 KB at 256 dimensions
     if (p.dims % 4 == 0 && ((uintptr_t)out & 15) == 0)
-        k_points_net<KIND, FMT, true><<<grid, 256, smem, s>>>(p, first, count, out);
+        k_points_net<KIND, FMT, true><<<grid, 256, smem, s>>>(p, first, count, out, parts);
     else
-        k_points_net<KIND, FMT, false><<<grid, 256, smem, s>>>(p, first, count, out);
+        k_points_net<KIND, FMT, false><<<grid, 256, smem, s>>>(p, first, count, out, parts);
 }
 
 template <int FMT>
@@ -263,7 +297,13 @@ static cudaError_t launch_points(const PointsP &p, uint64_t first, uint64_t coun
             p, first, count, out, (uint32_t)tile, p.dims % 4 == 0 && ((uintptr_t)out & 15) == 0);
         break;
     }
-    default: k_points_digits<FMT><<<grid_for(count * (uint64_t)p.dims), 256, 0, s>>>(p, first, count, out); break;
+    case QMCRT_HALTON:
+        k_points_digits<QMCRT_HALTON, FMT><<<grid_for(count * (uint64_t)p.dims), 256, 0, s>>>(p, first, count, out);
+        break;
+    case QMCRT_HAMMERSLEY:
+        k_points_digits<QMCRT_HAMMERSLEY, FMT><<<grid_for(count * (uint64_t)p.dims), 256, 0, s>>>(p, first, count, out);
+        break;
+    default: k_points_digits<QMCRT_FAURE, FMT><<<grid_for(count * (uint64_t)p.dims), 256, 0, s>>>(p, first, count, out);
     }
     return cudaGetLastError();
 }
