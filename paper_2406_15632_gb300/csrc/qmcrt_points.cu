@@ -1,6 +1,8 @@
 // qmcrt_points.cu -- point-set generation (Sec. 3.1), the final image reduction
 // (Sec. 3.6: sums of all replicas, in units of the source luminosity) and the padded
 // copy of a density grid.
+#include <algorithm>
+
 #include "qmcrt_device.cuh"
 
 namespace qmcrt {
@@ -224,41 +226,56 @@ __global__ void __launch_bounds__(256) k_image_reduce(const void *acc, int mode,
     }
 }
 
-// Copy of a grid with `pad` layers of sentinel cells on every side, a warp per row of the
-// padded grid (rows and their sources found once a row: a division a cell and 4-byte
-// accesses took 77 us at 256^3, this 24; 22 at the copy rate).  Interior: the density,
-// with empty, negative and NaN cells as +0 (no sign bit); padding: the sentinel -0.0, whose
-// sign bit ends a padded walk.  VEC: 16-byte accesses, for rows and padding of whole vectors.
-template <bool VEC>
+// Copy of a grid with `pad` layers of sentinel cells on every side.  Interior: the density, with
+// empty, negative and NaN cells as +0 (no sign bit); padding: the sentinel -0.0, whose sign bit
+// ends a padded walk.  V: float4 for rows and padding of whole vectors, else float.  Bound by the
+// copy: a thread walks the padded array at the grid's stride and carries its place along, rows of any
+// length alike, four loads ahead.  A call at 256^3, and on the 17-cell rows of 1 x 1 x 10^6: 79 and 933 us
+// with a division an element and 4-byte accesses, 31 and 2150 with a warp a row, 25 and 165 so.
+constexpr int PAD_BATCH = 4;  // loads in flight a thread
+template <class V>
+__device__ __forceinline__ V edge_cells();
+template <>
+__device__ __forceinline__ float edge_cells<float>() { return -0.0f; }
+template <>
+__device__ __forceinline__ float4 edge_cells<float4>() { return make_float4(-0.0f, -0.0f, -0.0f, -0.0f); }
+__device__ __forceinline__ float clean_cells(float v) { return v > 0.0f ? v : 0.0f; }
+__device__ __forceinline__ float4 clean_cells(float4 v)
+{
+    return make_float4(clean_cells(v.x), clean_cells(v.y), clean_cells(v.z), clean_cells(v.w));
+}
+
+template <class V>
 __global__ void __launch_bounds__(256) k_pad_grid(const float *__restrict__ k, int nx, int ny, int nz, int pad,
                                                  float *__restrict__ out)
 {
-    const int px = nx + 2 * pad, py = ny + 2 * pad, pz = nz + 2 * pad;
-    const long long rows = (long long)py * pz;
-    const int lane = threadIdx.x & 31;
-    auto clean = [](float v) { return v > 0.0f ? v : 0.0f; };
-    for (long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * 8) {
-        const int z = (int)(r / py) - pad, y = (int)(r % py) - pad;
-        const bool in = z >= 0 && z < nz && y >= 0 && y < ny;
-        const float *src = k + ((long long)z * ny + y) * nx;  // read only where the row is in the grid
-        float *dst = out + r * px;
-        if (VEC) {
-            const float4 edge = make_float4(-0.0f, -0.0f, -0.0f, -0.0f);
-            for (int v = lane; v < px / 4; v += 32) {
-                const int x = 4 * v - pad;
-                float4 q = edge;
-                if (in && x >= 0 && x < nx) {
-                    q = __ldg(reinterpret_cast<const float4 *>(src + x));
-                    q = make_float4(clean(q.x), clean(q.y), clean(q.z), clean(q.w));
-                }
-                reinterpret_cast<float4 *>(dst)[v] = q;
-            }
-        } else {
-            for (int c = lane; c < px; c += 32) {
-                const int x = c - pad;
-                dst[c] = in && x >= 0 && x < nx ? clean(__ldg(src + x)) : -0.0f;
-            }
+    constexpr unsigned W = sizeof(V) / sizeof(float);  // cells of an element
+    const unsigned ux = (unsigned)(nx + 2 * pad) / W, py = ny + 2 * pad, pz = nz + 2 * pad;
+    const unsigned stride = gridDim.x * blockDim.x, total = ux * py * pz;  // a padded grid holds at most 2^31 cells
+    const unsigned sr = stride / ux, sx = stride - sr * ux, sz = sr / py, sy = sr - sz * py;
+    unsigned e = blockIdx.x * blockDim.x + threadIdx.x, r = e / ux, x = e - r * ux, z = r / py, y = r - z * py;
+    while (e < total) {
+        V v[PAD_BATCH];
+        unsigned at[PAD_BATCH];
+#pragma unroll
+        for (int b = 0; b < PAD_BATCH; ++b) {
+            const unsigned cx = x * W - pad, cy = y - pad, cz = z - pad;  // beyond the grid: large
+            const bool in = cx < (unsigned)nx && cy < (unsigned)ny && cz < (unsigned)nz;  // beyond the array: not
+            v[b] = edge_cells<V>();
+            if (in) v[b] = clean_cells(__ldg(reinterpret_cast<const V *>(k + ((long long)cz * ny + cy) * nx + cx)));
+            at[b] = e;
+            e += stride;
+            x += sx;
+            const unsigned c = x >= ux;
+            x -= c * ux;
+            y += sy + c;
+            const unsigned d = y >= py;
+            y -= d * py;
+            z += sz + d;
         }
+#pragma unroll
+        for (int b = 0; b < PAD_BATCH; ++b)
+            if (at[b] < total) reinterpret_cast<V *>(out)[at[b]] = v[b];
     }
 }
 
@@ -317,14 +334,22 @@ cudaError_t launch_generate_points(const PointsP &p, uint64_t first, uint64_t co
     return launch_points<QMCRT_FMT_F64>(p, first, count, out, s);
 }
 
+// Blocks of 256 threads with PAD_BATCH elements each, at most per_sm a multiprocessor: single cells at 32
+// (four rounds of resident ones; the set-up's divisions weigh on more: 255^3 33 us, 41 at 128), whole
+// vectors at 512 (padding is written faster so: 1 x 4096^2 166 us, 191 at 32).
+static unsigned pad_blocks(uint64_t elements, unsigned per_sm)
+{
+    const uint64_t b = (elements + 256 * PAD_BATCH - 1) / (256 * PAD_BATCH);
+    return (unsigned)std::min<uint64_t>(b, 152ull * per_sm);
+}
+
 cudaError_t launch_pad_grid(const float *k, int nx, int ny, int nz, int pad, float *out, cudaStream_t s)
 {
-    const uint64_t rows = (uint64_t)(ny + 2 * pad) * (nz + 2 * pad);
-    const unsigned grid = (unsigned)((rows + 7) / 8 < 152 * 16 ? (rows + 7) / 8 : 152 * 16);
+    const uint64_t cells = (uint64_t)(nx + 2 * pad) * (ny + 2 * pad) * (nz + 2 * pad);
     if (nx % 4 == 0 && pad % 4 == 0 && (((uintptr_t)k | (uintptr_t)out) & 15) == 0)
-        k_pad_grid<true><<<grid, 256, 0, s>>>(k, nx, ny, nz, pad, out);
+        k_pad_grid<float4><<<pad_blocks(cells / 4, 512), 256, 0, s>>>(k, nx, ny, nz, pad, out);
     else
-        k_pad_grid<false><<<grid, 256, 0, s>>>(k, nx, ny, nz, pad, out);
+        k_pad_grid<float><<<pad_blocks(cells, 32), 256, 0, s>>>(k, nx, ny, nz, pad, out);
     return cudaGetLastError();
 }
 
