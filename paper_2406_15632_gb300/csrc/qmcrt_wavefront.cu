@@ -398,7 +398,13 @@ cudaError_t launch_wave(TraceP<T> P, void *ws, uint64_t cap, int sms, cudaStream
     cudaError_t e = cudaMemsetAsync(W.count, 0, WV_TAIL_BYTES, s);
     if (e == cudaSuccess && P.max_orders > 1) e = cudaMemsetAsync(W.hist, 0, (size_t)buckets * sizeof(uint32_t), s);
     if (e != cudaSuccess) return e;
-    if (P.med.kind == QMCRT_MEDIUM_GRID && P.med.pad && P.med.inv_half[0] > 0.0f) {
+    // The support costs a read of the grid, 200 us and the caches at 512^3 (6 us at 256^3), which few
+    // packets do not pay for.  512^3 clumpy envelope, us without and with it: 2 orders of 2^10 packets
+    // 452 / 524, of 2^12 591 / 561; 5 of 2^8 935 / 1175, of 2^10 1512 / 1314; 1 of 2^16 294 / 327; 256^3: 2
+    // of 2^8 138 / 135, 1 of 2^14 72 / 77, of 2^16 90 / 82.
+    const uint64_t cells = (uint64_t)P.med.n[0] * P.med.n[1] * P.med.n[2];
+    const bool few = P.max_orders > 1 ? P.count * (P.max_orders - 1) < cells >> 16 : P.count < cells >> 9;
+    if (P.med.kind == QMCRT_MEDIUM_GRID && P.med.pad && P.med.inv_half[0] > 0.0f && !few) {
         uint32_t *support = (uint32_t *)(W.count + 66);
         k_support<T><<<(unsigned)std::max(1, sms * 8), 256, 0, s>>>(P.med, support_scale2(P.med), support);
         P.med.support = (const float *)support;

@@ -102,3 +102,18 @@ def test_small_batches_with_and_without_the_cut(Q, sizes):
     torch.cuda.synchronize()
     assert torch.equal(got, b.accum)
     assert bool((got != 0).any()) == (max(sizes) > 0)
+
+
+@pytest.mark.parametrize("orders,n", [(2, 3), (2, 4), (2, 5), (3, 1), (3, 2), (9, 40)])
+def test_short_wavefronts_with_and_without_the_cut(Q, orders, n):
+    """Counts on both sides of the one from which a run looks for the support, of a 64^3 grid."""
+    import torch
+
+    p = _problem("unit", max_orders=orders, per_order=True)
+    p = p.replace(grid=np.repeat(np.repeat(np.repeat(p.grid, 3, 0), 3, 1), 3, 2)[4:68, 4:68, 4:68].copy())
+    sc = Q.Scene(p, sky=0)
+    a, b = sc.accum_buffer("i64"), sc.accum_buffer("i64")
+    sc.trace(7, n, a, frac_bits=36)
+    sc.trace_wavefront(7, n, b, sc.wavefront_workspace(n), frac_bits=36)
+    torch.cuda.synchronize()
+    assert torch.equal(a, b)
