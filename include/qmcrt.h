@@ -278,7 +278,7 @@ int qmcrt_trace_batch(const qmcrt_medium *medium, const qmcrt_source *source, co
 int qmcrt_batch_reduce(const qmcrt_image *image, const qmcrt_instance *d_instances, int32_t n_instances, int32_t nx,
                        int32_t ny, double *d_out, void *stream);
 
-/* ---- tensor-core GEMM (building block of the learned proposal) ---- */
+/* ---- tensor-core GEMM ---- */
 typedef struct qmcrt_gemm_epilogue {
     uint32_t struct_size;
     int32_t relu;            /* max(0, .) after the bias */
@@ -296,8 +296,7 @@ typedef struct qmcrt_gemm_epilogue {
  * qmcrt_gemm_bf16 -- D[M][N] = A[M][K] . B[N][K]^T on the tensor cores (BF16 inputs, FP32
  * accumulation), then the epilogue (bias, ReLU, ReLU mask, FP32 / BF16 / transposed
  * BF16 outputs).  A, B: device bf16, row-major, K contiguous, 16-byte aligned; the mask
- * and the FP32 / BF16 outputs 16-byte aligned too.  The paper has no counterpart; it is
- * the building block of the learned warp's network.
+ * and the FP32 / BF16 outputs 16-byte aligned too.  The paper has no counterpart.
  * Errors: INVALID_ARG (NULL pointers, M < 1, N not 32/64/128, K not a positive multiple
  * of 32, ldt < M, bias with k_splits > 1, misaligned pointers), CUDA.
  */
@@ -326,7 +325,8 @@ typedef struct qmcrt_warp {
                             bounds |dx/du| by mix^-3 */
     float *d_params;     /* device FP32 [QMCRT_WARP_PARAMS] */
     void *d_weights;     /* device bf16 [QMCRT_WARP_BF16_WEIGHTS] (refreshed by qmcrt_warp_sync) */
-    void *d_weights_t;   /* device bf16 [QMCRT_WARP_BF16_WEIGHTS], the transposes */
+    void *d_weights_t;   /* device bf16 [QMCRT_WARP_BF16_WEIGHTS], the transposes (written for the
+                            caller: the library's kernels read d_weights both ways) */
     int32_t *d_error;    /* device int or NULL: set to 1 if a tensor-core wait gives up */
 } qmcrt_warp;
 
@@ -336,7 +336,8 @@ typedef struct qmcrt_adam {
     double lr, beta1, beta2, eps;
 } qmcrt_adam;
 
-/* Device workspace bytes for the warp calls processing up to `rows` samples per pass. */
+/* Device workspace bytes for the warp calls processing up to `rows` samples per pass (3328 a row;
+ * the rows that fit set the length of a pass, and with it the order in which qmcrt_warp_grad sums). */
 uint64_t qmcrt_warp_workspace_bytes(uint64_t rows);
 
 /* Refresh the bf16 weight copies (as is and transposed) from the FP32 parameters. */
@@ -475,7 +476,7 @@ int qmcrt_image_reduce(const qmcrt_image *image, int32_t nx, int32_t ny, int32_t
  * texel's centre ray (alpha: the texel's angular radius), hence, while that is at most D
  * smallest cell edges (D = 1 + ceil(radius / h_min)), within D cells of the centre ray's
  * cell at equal t; the map holds the integral, along the centre ray, of the grid maximised
- * over (2 D + 1)^3 neighbourhoods (times 1 + 1e-6).  A texel whose cone is wider than that
+ * over (2 D + 1)^3 neighbourhoods (times 1 + 1e-4).  A texel whose cone is wider than that
  * (too coarse a map for the grid: m below about 1.2 x the cells per axis) holds +inf.
  * d_k: device [nz][ny][nx] grid (not padded); lo, hi: host [3], the grid box; d_workspace:
  * device, 256-byte aligned, >= qmcrt_sky_workspace_bytes (two grids grown by D layers).

@@ -548,9 +548,9 @@ __device__ __forceinline__ bool grid_walk(const MediumP<T> &G, const T p[3], con
 // negative zero (qmcrt_pad_grid writes +0 for empty, negative or NaN cells).  The walk
 // needs no per-axis cell counters: a batch of WALK_UNROLL cells is stepped blindly (at
 // most WALK_UNROLL cells past the box, still inside the padding), a sentinel adds
-// L * (-0) = -0, nothing, and the walk ends after the first batch in which a loaded
-// value has its sign bit set.  The box is convex and axis-aligned, so once a step
-// leaves it along any axis every later cell of the ray is outside too.  The optical
+// L * (-0) = -0, nothing, and the walk ends after the first batch whose last value
+// has its sign bit set.  The box is convex and axis-aligned, so once a step leaves it along
+// any axis every later cell of the ray, the batch's last among them, is outside too.  The optical
 // depths of a batch are summed in order and the batch sum enters the compensated
 // total; the march tests the batch sum against the remaining depth and only then
 // looks for the stopping cell inside the batch.
@@ -847,17 +847,7 @@ __device__ __forceinline__ bool padded_march(const float *__restrict__ K, Padded
     return false;
 }
 
-// The same walk over a padded grid (QMCRT pad >= WALK_UNROLL): the grid is
-// surrounded by `pad` layers of sentinel cells holding -0.0, and the interior holds no
-// negative zero (qmcrt_pad_grid writes +0 for empty, negative or NaN cells).  The walk
-// needs no per-axis cell counters: a batch of WALK_UNROLL cells is stepped blindly (at
-// most WALK_UNROLL cells past the box, still inside the padding), a sentinel adds
-// L * (-0) = -0, nothing, and the walk ends after the first batch in which a loaded
-// value has its sign bit set.  The box is convex and axis-aligned, so once a step
-// leaves it along any axis every later cell of the ray is outside too.  The optical
-// depths of a batch are summed in order and the batch sum enters the compensated
-// total; the march tests the batch sum against the remaining depth and only then
-// looks for the stopping cell inside the batch.
+// The walk over a padded grid as grid_walk states it: the depth to the edge, or the march to target_raw.
 template <class T, bool TARGET>
 __device__ __forceinline__ bool grid_walk_padded(const MediumP<T> &G, const T p[3], const T d[3], const T r[3],
                                                  T target_raw, T &tau_raw, T &t_out)

@@ -5,9 +5,9 @@
 // tiles of the minibatch: features, the four layers forward, the loss gradient of the logits,
 // the three layers backward, with every activation and backward signal of the tile in shared
 // memory (F 16 KB, H1-H3 32 KB each, the logits' gradient 8 KB) and the products' accumulator
-// in TMEM.  The weight gradients dW[l] = dP[l]^T H[l] are summed over all the tiles of a CTA in
-// TMEM (352 columns beside the 128 of the accumulator) and leave once, at its end, as vector
-// reductions into the caller's gradient; bias gradients are summed in registers.
+// in TMEM.  The weight gradients dW[l] = dP[l]^T H[l] are summed over the tiles of a slice of about
+// 512 rows in TMEM (352 columns beside the 128 of the accumulator) and leave at its end as vector
+// reductions into the caller's gradient; bias gradients are summed in registers over all of them.
 //
 // No operand is ever stored twice: a tile [rows][columns] lies in the canonical no-swizzle
 // layout (8 x 16-byte core matrices), which the tensor core reads with its rows as M or N and
@@ -17,7 +17,7 @@
 // backward.  A backward signal replaces the activation it was masked with.
 //
 // What bounds it: the chain of a tile, eight products of some hundred cycles each behind an
-// epilogue of 8 warps (TMEM read, bias or mask, bf16 packing).  A layer-by-layer form (14 GEMMs
+// epilogue of 16 warps (TMEM read, bias or mask, bf16 packing).  A layer-by-layer form (14 GEMMs
 // through HBM, 8 split-K GEMMs, feature, loss and row-sum kernels) moved 0.5 GB and took 560 us
 // for 2^16 rows; this 110 us (10 us a tile, two slices a CTA).
 //

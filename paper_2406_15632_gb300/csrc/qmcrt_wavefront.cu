@@ -377,8 +377,9 @@ WaveWork<T> carve(void *ws, uint64_t cap)
 
 // Bits of the key for n packets.  20-order clumpy envelope, 16^3 position cells x 32 x 64 direction
 // bins against 8^3 cells with the same bins: 20.9 / 21.3 ms at 2^22 packets, 6.51 / 6.40 at
-// 2^20, 2.75 / 2.69 at 2^18, 1.79 / 1.73 at 2^16, and on a 32^3 grid 5.49 / 5.18 at 2^20; fewer
-// direction bins lose at every size but the smallest, where no split matters (2^12: 1.15 ms).
+// 2^20, 2.75 / 2.69 at 2^18, 1.79 / 1.73 at 2^16, and on a 32^3 grid 5.49 / 5.18 at 2^20.  Now, on 128^3:
+// 15.28 / 15.58 at 2^22, 8.29 / 8.36 at 2^21, 6.36 / 6.38 at 2^20.5, 4.73 / 4.70 at 2^20; on 48^3 the coarse
+// key is 4 to 6 % faster at any size up to 2^22.  Fewer direction bins lose at every size but the smallest, where no split matters (2^12: 1.15 ms).
 // With a three-launch scan, clears and copies an order took up to 150 us on the buckets alone,
 // and the same runs 22.3, 8.1, 4.4 and 3.3 ms.
 WaveKey wave_bits(uint64_t n, uint64_t queue_bytes)
