@@ -330,7 +330,9 @@ int fill_trace(const qmcrt_medium *md, const qmcrt_source *src, const qmcrt_dust
         // scale^2 is about the shortest half edge (support_batches).  No cut (inv_half = 0) beyond 1e24
         // or below 1e-24 units, in a box of edges a factor of 1000 apart, or far from the origin, where
         // the float rounding of a position (a few roundings of |lo| or |hi|) would outgrow its room.
-        const double scale = std::exp2(std::floor(0.5 * std::log2(0.5 * edge)));
+        int e2;
+        std::frexp(edge, &e2);
+        const double scale = std::ldexp(1.0, (e2 - 1) / 2);
         const bool cut = edge > 1e-24 && edge < 1e24 && longest < 1000.0 * edge && far < 2.5;
         for (int a = 0; a < 3; ++a) P.med.inv_half[a] = cut ? (float)(2.0 * scale / (md->hi[a] - md->lo[a])) : 0.0f;
         if (md->pad != 0 && md->pad < QMCRT_MIN_PAD)
