@@ -35,12 +35,13 @@ __device__ __forceinline__ uint64_t instance_tiles(const qmcrt_instance &I, int 
 // holds the medium's support (cleared here), with which first walks end where they leave the
 // medium: 15.1 -> 14.3 ms for 24 instances of the 256^3 finite-star disk, 38 M packets.  The cut
 // costs a read of the grid, which few packets do not pay for: it is left out (the support set
-// to everything) below cells / 2048 packets, unless an instance has 8192, whose longest walks
-// then count.  Start to end in us, without and with it: 256^3 with 2^10 packets 209 / 241, 2^12 258 / 281,
+// to everything) below `enough` packets, cells / 2048 (FP64, whose walks are dearer: cells / 131072), unless
+// an instance has 8192, whose longest walks then count.  Start to end in us, without and with it: 256^3 with 2^10 packets 209 / 241, 2^12 258 / 281,
 // 2^13 340 / 319, 24 x 2^8 147 / 177, 24 x 2^10 361 / 346; 512^3 with 2^10 498 / 779, 2^13 843 / 806,
-// 24 x 2^10 644 / 809, 24 x 2^12 1010 / 948.  One block of 1024 threads.
+// 24 x 2^10 644 / 809, 24 x 2^12 1010 / 948; FP64, 128^3 with 2^9 357 / 334, 400^3 with 2^7 324 / 441, with
+// 2^9 844 / 852, with 2^10 1728 / 1675.  One block of 1024 threads.
 __global__ void __launch_bounds__(1024) k_batch_plan(const qmcrt_instance *__restrict__ inst, int n, int m_cap,
-                                                    uint64_t tile_packets, uint64_t cells,
+                                                    uint64_t tile_packets, uint64_t enough,
                                                     unsigned long long *__restrict__ ws)
 {
     __shared__ unsigned long long part[1024];
@@ -79,7 +80,7 @@ __global__ void __launch_bounds__(1024) k_batch_plan(const qmcrt_instance *__res
     if (t == 1023) ws[1 + n] = part[1023];
     if (t == 0) {
         ws[0] = 0ull;
-        const bool few = s_most < 8192 && s_all < cells / 2048;  // at most 2^20
+        const bool few = s_most < 8192 && s_all < enough;  // at most 2^20
         const unsigned long long none = __float_as_uint(SUPPORT_ALL);
         ws[1] = few ? none << 32 | none : 0ull;
     }
@@ -216,8 +217,8 @@ template <class T>
 static cudaError_t launch_batch(TraceP<T> p, const NetTables &tab, const qmcrt_instance *inst, int n_inst,
                                 unsigned long long *ws, int block, int ctas, int per_thread, cudaStream_t s)
 {
-    const uint64_t cells = (uint64_t)p.med.n[0] * p.med.n[1] * p.med.n[2];
-    k_batch_plan<<<1, 1024, 0, s>>>(inst, n_inst, tab.m_cap, (uint64_t)block * per_thread, cells, ws);
+    const uint64_t enough = (uint64_t)p.med.n[0] * p.med.n[1] * p.med.n[2] / (sizeof(T) == 8 ? 131072 : 2048);
+    k_batch_plan<<<1, 1024, 0, s>>>(inst, n_inst, tab.m_cap, (uint64_t)block * per_thread, enough, ws);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (p.med.kind == QMCRT_MEDIUM_GRID && p.med.pad && p.med.inv_half[0] > 0.0f) {

@@ -402,8 +402,8 @@ cudaError_t launch_wave(TraceP<T> P, void *ws, uint64_t cap, int sms, cudaStream
     // The support costs a read of the grid, 200 us and the caches at 512^3 (6 us at 256^3), which few
     // packets do not pay for.  512^3 clumpy envelope, us without and with it: 2 orders of 2^10 packets
     // 452 / 524, of 2^12 591 / 561; 5 of 2^8 935 / 1175, of 2^10 1512 / 1314; 1 of 2^16 294 / 327; 256^3: 2
-    // of 2^8 138 / 135, 1 of 2^14 72 / 77, of 2^16 90 / 82.
-    const uint64_t cells = (uint64_t)P.med.n[0] * P.med.n[1] * P.med.n[2];
+    // of 2^8 138 / 135, 1 of 2^14 72 / 77, of 2^16 90 / 82.  FP64 walks are dearer: a 64th of the packets.
+    const uint64_t cells = ((uint64_t)P.med.n[0] * P.med.n[1] * P.med.n[2]) >> (sizeof(T) == 8 ? 6 : 0);
     const bool few = P.max_orders > 1 ? P.count * (P.max_orders - 1) < cells >> 16 : P.count < cells >> 9;
     if (P.med.kind == QMCRT_MEDIUM_GRID && P.med.pad && P.med.inv_half[0] > 0.0f && !few) {
         uint32_t *support = (uint32_t *)(W.count + 66);

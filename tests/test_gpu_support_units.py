@@ -83,8 +83,9 @@ def test_box_beside_the_star(Q, precision):
     assert bool((a[:, 1:] != 0).any())
 
 
-@pytest.mark.parametrize("sizes", [(1,), (2047,), (2048,), (100, 8191), (8192, 0, 5), (0, 0), (700, 700, 700)])
-def test_small_batches_with_and_without_the_cut(Q, sizes):
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+@pytest.mark.parametrize("sizes", [(1,), (5,), (6,), (7,), (2047,), (2048,), (100, 8191), (8192, 0, 5), (0, 0), (700, 700, 700)])
+def test_small_batches_with_and_without_the_cut(Q, sizes, precision):
     """Batches on both sides of the size from which the support is looked for, one after another in one
     workspace."""
     import torch
@@ -93,7 +94,7 @@ def test_small_batches_with_and_without_the_cut(Q, sizes):
     sc = Q.Scene(p)
     inst = [S.Instance(theta_obs=0.3 * k, albedo=0.7, g=0.4, kscale=0.5 + k, n_packets=n, first_index=9)
             for k, n in enumerate(sizes)]
-    b = Q.Batch(p, inst, frac_bits=36, scene=sc)
+    b = Q.Batch(p, inst, frac_bits=36, scene=sc, precision=precision)
     for _ in range(2):
         b.run()
         got = b.accum.clone()
